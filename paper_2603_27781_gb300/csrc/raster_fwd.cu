@@ -1,7 +1,7 @@
 // Forward blend (GS3LAM Eq. 4-7 and 10): one CTA per 16x16 tile, NP pixels per
 // thread.  Splats of the tile are staged 128 at a time in shared memory (one
 // record per thread load) and read back as broadcasts; a warp tests 32 splats at
-// a time (one per lane, one ballot) for whether their alpha >= alpha_min region
+// a time (one per lane, one ballot) for whether their alpha >= alpha_min ellipse
 // reaches its pixel box, and walks only those that do; every pixel walks the
 // rest front to back and stops at the T_min threshold; the CTA leaves as soon
 // as all of its pixels are done.  With a blend mask, each warp also records, per
@@ -20,6 +20,137 @@ constexpr int fwd_min_blocks(int D, int NP) {
     return NP == 1 ? (D == 0 ? 8 : D <= 4 ? 6 : D <= 16 ? 5 : 3) : NP == 2 ? (D <= 16 ? 6 : 4) : 6;
 }
 
+// A staged splat is one record of 3 + D / 4 16-byte words: geometry (two), colour and depth, the
+// features.  One base address serves all of a splat's reads, and the odd word counts of D = 0, 8, 16
+// and 32 keep eight threads that write neighbouring records in different banks.
+template <int D> constexpr int kRecWords = 3 + D / 4;
+
+__device__ __forceinline__ SplatGeo geo_of(const float4 *rec) {
+    const float4 a = rec[0], b = rec[1];
+    return SplatGeo{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+}
+__device__ __forceinline__ void put_geo(float4 *rec, const SplatGeo &s) {
+    rec[0] = make_float4(s.u, s.v, s.ulo, s.vlo);
+    rec[1] = make_float4(s.qa, s.qb, s.qc, s.o);
+}
+
+// The pixels of one thread while they are blended: position, transmittance, the alpha below which
+// a splat is skipped (alpha_min, and infinity once the pixel is done or lies outside the image) and
+// the blended sums.  The sums are kept as packed pairs of channels ((r, g), (b, depth), the
+// features), which match the 16-byte words of the staged records, so a splat costs (4 + D) / 2
+// packed multiply-adds per pixel instead of 4 + D scalar ones, with the same rounding.
+//
+// The kernel is bound by instruction issue (74 % of cycles at D = 16) and by the latency of the
+// staging between its barriers.  One base address per record, packed multiply-adds and the exact
+// ellipse test alone (the rectangle test before it cost a logarithm, two roots and two divisions per
+// staged splat and culled almost nothing more) took the forward from 0.266 to 0.246 ms (room, 1M
+// Gaussians, D = 16, 1200x680), 0.230 to 0.190 ms (1M, D = 32, 640x480), 4.33 to 3.26 ms (2M, D = 32,
+// 16-bit storage, 8 keyframes) and 0.107 to 0.075 ms (300k, D = 8, 811x607), bit-identical.  Measured
+// and slower: the next batch's records copied (cp.async) into a second buffer while the current one
+// is walked (0.339 ms with 128-splat batches, 0.282 with 64: the second buffer takes the L1 that
+// serves the gathers of neighbouring tiles), and the box tests done once by the staging thread for
+// all four warps (0.262 against 0.237 ms: they then sit between the loads and the barrier).
+template <int D, int NP>
+struct BlendPixels {
+    using SH = Shape<NP, true>;  // horizontal pixel pairs
+    static constexpr int NL = SH::PIX_GROUPS ? NP : 1;  // mask bit registers per thread
+    static constexpr int D4 = D / 4, F4 = D4 > 0 ? D4 : 1;
+    float pxc[NP], pyc[NP], T[NP], lim[NP], as[NP];
+    float2 acc[NP][2], af[NP][2 * F4];
+    int last[NP], blended[NP];
+
+    __device__ __forceinline__ void init(const ViewTable &vt, const Params &prm, int v, int tx, int ty, int tid) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            int lx, ly;
+            SH::pixel(tid, p, lx, ly);
+            const int px = tx * kTile + lx, py = ty * kTile + ly;
+            pxc[p] = (float)px + 0.5f;
+            pyc[p] = (float)py + 0.5f;
+            T[p] = 1.f;
+            lim[p] = px < vt.W[v] && py < vt.H[v] ? prm.alpha_min : INFINITY;
+            as[p] = 0.f;
+            acc[p][0] = acc[p][1] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < 2 * F4; ++q) af[p][q] = make_float2(0.f, 0.f);
+            last[p] = blended[p] = 0;
+        }
+    }
+    __device__ __forceinline__ bool all_done() const {
+        bool a = true;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) a = a && lim[p] == INFINITY;
+        return a;
+    }
+    // Blends one staged splat (its record, list position pos, mask bit `bit`) into the thread's pixels.
+    template <bool CNT>
+    __device__ __forceinline__ void blend(const Params &prm, const float4 *rec, int pos, uint32_t bit,
+                                          uint32_t (&lbits)[NL]) {
+        const SplatGeo s = geo_of(rec);
+        float wgt[NP];
+        bool any = false;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const PairEval e = eval_pair(s, pxc[p], pyc[p], lim[p], prm.alpha_max);
+            const float Tn = T[p] * (1.f - e.alpha);
+            const bool stop = !e.skip && Tn < prm.T_min;
+            const bool b = !e.skip && !stop;
+            lim[p] = stop ? INFINITY : lim[p];
+            wgt[p] = b ? e.alpha * T[p] : 0.f;
+            T[p] = b ? Tn : T[p];
+            last[p] = b ? pos : last[p];
+            if constexpr (CNT) blended[p] += b ? 1 : 0;
+            any = any || b;
+            if (SH::PIX_GROUPS) lbits[p % NL] |= b ? bit : 0u;
+        }
+        if (!SH::PIX_GROUPS) lbits[0] |= any ? bit : 0u;
+        if (!any) return;
+        const float4 c = rec[2];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const float2 w = make_float2(wgt[p], wgt[p]);
+            as[p] += wgt[p];
+            acc[p][0] = fma2(w, make_float2(c.x, c.y), acc[p][0]);
+            acc[p][1] = fma2(w, make_float2(c.z, c.w), acc[p][1]);
+        }
+#pragma unroll
+        for (int q = 0; q < D4; ++q) {
+            const float4 f = rec[3 + q];
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const float2 w = make_float2(wgt[p], wgt[p]);
+                af[p][2 * q] = fma2(w, make_float2(f.x, f.y), af[p][2 * q]);
+                af[p][2 * q + 1] = fma2(w, make_float2(f.z, f.w), af[p][2 * q + 1]);
+            }
+        }
+    }
+    __device__ __forceinline__ void write(const ViewTable &vt, const Params &prm, int v, int tx, int ty, int tid, int64_t P,
+                                          float *o_rgb, float *o_depth, float *o_sil, float *o_feat, float *o_T,
+                                          int32_t *o_nc, int32_t *o_nb) const {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            int lx, ly;
+            SH::pixel(tid, p, lx, ly);
+            const int px = tx * kTile + lx, py = ty * kTile + ly;
+            if (px >= vt.W[v] || py >= vt.H[v]) continue;
+            const int64_t pix = vt.pix_off[v] + (int64_t)py * vt.W[v] + px;
+            o_rgb[pix] = acc[p][0].x + T[p] * prm.bg[0];
+            o_rgb[P + pix] = acc[p][0].y + T[p] * prm.bg[1];
+            o_rgb[2 * P + pix] = acc[p][1].x + T[p] * prm.bg[2];
+            o_depth[pix] = acc[p][1].y;
+            o_sil[pix] = as[p];
+#pragma unroll
+            for (int q = 0; q < D / 2; ++q) {
+                o_feat[(2 * q) * P + pix] = af[p][q].x;
+                o_feat[(2 * q + 1) * P + pix] = af[p][q].y;
+            }
+            o_T[pix] = T[p];
+            o_nc[pix] = last[p];
+            if (o_nb) o_nb[pix] = blended[p];
+        }
+    }
+};
+
 // One 16x16 tile gt of the blend, by the whole CTA (every exit is uniform over the CTA), staging
 // BATCH splats per round; with CNT it also counts each pixel's blended splats (o_nb).
 template <int D, int NP, typename RT, typename FT, int BATCH, bool CNT>
@@ -30,179 +161,85 @@ __device__ __forceinline__ void fwd_tile(
     float *o_sil, float *o_feat, float *o_T, int32_t *o_nc, int32_t *o_nb, uint32_t *bmask, int64_t bm_stride,
     const int gt, int32_t *status, int64_t capacity) {
     using SH = Shape<NP, true>;  // horizontal pixel pairs
-    constexpr int NT = SH::THREADS;
+    constexpr int NT = SH::THREADS, REC = kRecWords<D>, D4 = D / 4;
     constexpr int NL = SH::PIX_GROUPS ? NP : 1;  // mask bit registers per thread
-    constexpr int D4 = D / 4, DD = D > 0 ? D : 1;
-    // the batch's records: geometry, culling extents, colour and depth, features
-    constexpr int batch = BATCH;
-    __shared__ SplatGeo s_geo[BATCH];
-    __shared__ float2 s_ext[BATCH];
-    __shared__ float4 s_cull[BATCH];
-    __shared__ float4 s_rgbd[BATCH];
-    __shared__ float4 s_feat[BATCH * (D4 > 0 ? D4 : 1)];
+    __shared__ float4 s_rec[BATCH * REC];  // the batch's records
+    __shared__ float4 s_cull[BATCH];       // their culling constants
 
     if (gt < 0 || gt >= vt.tile_off[vt.n_views]) return;  // not a permutation of the tiles: leave the tile
     const int v = view_of_tile(vt, gt);
     const int t = gt - vt.tile_off[v];
     const int tx = t % vt.TX[v], ty = t / vt.TX[v];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint32_t start = ranges[2 * gt], end = ranges[2 * gt + 1];
     checked_range(start, end, capacity, status);
     const int64_t voff = (int64_t)v * vt.n;
     int bx0, by0;
-    SH::warp_origin(tid >> 5, bx0, by0);
+    SH::warp_origin(warp, bx0, by0);
     const float bcx = (float)(tx * kTile + bx0) + 0.5f * SH::BW, bcy = (float)(ty * kTile + by0) + 0.5f * SH::BH;
     const float hx = 0.5f * (SH::BW - 1), hy = 0.5f * (SH::BH - 1);
 
-    float pxc[NP], pyc[NP], T[NP], ar[NP], ag[NP], ab[NP], ad[NP], as[NP], af[NP][DD];
-    int last[NP], blended[NP];
-    bool inside[NP], done[NP];
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        int lx, ly;
-        SH::pixel(tid, p, lx, ly);
-        const int px = tx * kTile + lx, py = ty * kTile + ly;
-        inside[p] = px < vt.W[v] && py < vt.H[v];
-        done[p] = !inside[p];
-        pxc[p] = (float)px + 0.5f;
-        pyc[p] = (float)py + 0.5f;
-        T[p] = 1.f;
-        ar[p] = ag[p] = ab[p] = ad[p] = as[p] = 0.f;
-#pragma unroll
-        for (int d = 0; d < DD; ++d) af[p][d] = 0.f;
-        last[p] = blended[p] = 0;
-    }
-    auto all_done = [&]() {
-        bool a = true;
-#pragma unroll
-        for (int p = 0; p < NP; ++p) a = a && done[p];
-        return a;
-    };
-    // blend-mask bits: batches start on 32-instance boundaries, so each 32-splat
-    // chunk of a batch is one word of the mask; a lane ORs "my pixel(s) of group j
-    // blended splat k" into a register (one per group its pixels lie in) and the
-    // warp combines the lanes of each of its NP groups at the end of the chunk
-    const int warp = tid >> 5, lane = tid & 31;
-    auto flush = [&](const uint32_t (&lbits)[NL], uint32_t word_idx) {
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            const uint32_t mine =
-                SH::PIX_GROUPS ? lbits[j % NL] : ((SH::lanes_of_group(j) >> lane) & 1u ? lbits[0] : 0u);
-            const uint32_t word = __reduce_or_sync(0xffffffffu, mine);
-            if (lane == 0 && word) atomicOr(&bmask[(int64_t)SH::group(warp, j) * bm_stride + word_idx], word);
-        }
-    };
+    BlendPixels<D, NP> px;
+    px.init(vt, prm, v, tx, ty, tid);
 
     bool finished = false;
     // every warp stays in the batch loop (it stages splats and meets the CTA
     // barriers); a warp whose pixels are all done only skips the splat loop
-    for (uint32_t b0 = start & ~31u; b0 < end; b0 += batch) {
-        if (__syncthreads_count(!all_done()) == 0) break;
-        for (int i = tid; i < batch; i += NT) {
+    for (uint32_t b0 = start & ~31u; b0 < end; b0 += BATCH) {
+        if (__syncthreads_and(px.all_done())) break;
+        for (int i = tid; i < BATCH; i += NT) {
             const uint32_t j = b0 + i;
             if (j >= start && j < end) {
                 const uint32_t item = checked_item(vals[j], voff, vt.n, status);
                 const int64_t g = (int64_t)item - voff;
                 const float4 a = uvdo[item];
-                const float4 c = conic[item];
-                s_geo[i] = make_geo(a, uv_lo[item], c);
-                s_ext[i] = splat_extent(c, a.w, prm.alpha_min);
-                s_cull[i] = ellipse_cull(s_geo[i], prm.alpha_min);
-                s_rgbd[i] = load_rgbd(rgb, g, a.z);
+                const SplatGeo sg = make_geo(a, uv_lo[item], conic[item]);
+                float4 *rec = s_rec + i * REC;
+                put_geo(rec, sg);
+                s_cull[i] = ellipse_cull(sg, prm.alpha_min);
+                rec[2] = load_rgbd(rgb, g, a.z);
 #pragma unroll
-                for (int q = 0; q < D4; ++q) s_feat[i * D4 + q] = load_feat4(feat, g * D + 4 * q);
+                for (int q = 0; q < D4; ++q) rec[3 + q] = load_feat4(feat, g * D + 4 * q);
             }
         }
         __syncthreads();
-        const int k_lo = b0 < start ? (int)(start - b0) : 0;
-        const int nb = min((uint32_t)batch, end - b0);
-        for (int c0 = k_lo & ~31; c0 < nb && !finished; c0 += 32) {
+        for (int c0 = 0; c0 < BATCH && !finished; c0 += 32) {
+            // the chunk's splats that can reach the warp's box, lane k testing splat c0 + k
+            const uint32_t j = b0 + c0 + lane;
+            const float4 *chunk = s_rec + c0 * REC;
+            const bool reach = j >= start && j < end &&
+                               reaches_box_exact(geo_of(chunk + lane * REC), s_cull[c0 + lane], bcx, bcy, hx, hy);
+            uint32_t todo = __ballot_sync(0xffffffffu, reach);
+            if (todo == 0u) continue;
+            // blend-mask bits: batches start on 32-instance boundaries, so each 32-splat chunk is one
+            // word of the mask; a lane ORs "my pixel(s) of group j blended splat k" into a register
+            // (one per group its pixels lie in) and the warp combines the lanes of each of its NP
+            // groups at the end of the chunk
             uint32_t lbits[NL];
 #pragma unroll
-            for (int j = 0; j < NL; ++j) lbits[j] = 0u;
-            // the chunk's splats in [k_lo, nb) that can reach the warp's box, lane k - c0
-            // testing splat k
-            const int kl = c0 + lane;
-            bool reach = false;
-            if (kl >= k_lo && kl < nb) {
-                const SplatGeo sg = s_geo[kl];
-                reach = reaches_box(sg.u, sg.v, s_ext[kl], bcx, bcy, hx, hy) &&
-                        reaches_box_exact(sg, s_cull[kl], bcx, bcy, hx, hy);
-            }
-            uint32_t todo = __ballot_sync(0xffffffffu, reach);
+            for (int l = 0; l < NL; ++l) lbits[l] = 0u;
+            const int pos0 = (int)(b0 + c0 - start) + 1;
             for (int n_run = 0; todo; ++n_run) {
-                const int k = c0 + __ffs(todo) - 1;
+                const int k = __ffs(todo) - 1;
                 todo &= todo - 1;
                 // every 4th splat walked: are all of the warp's pixels done? (a later exit only
                 // runs splats whose pairs blend nothing)
-                if ((n_run & 3) == 0 && __all_sync(0xffffffffu, all_done())) { finished = true; break; }
-                const SplatGeo s = s_geo[k];
-                float al[NP];
-                bool ok[NP];
+                if ((n_run & 3) == 0 && __all_sync(0xffffffffu, px.all_done())) { finished = true; break; }
+                px.template blend<CNT>(prm, chunk + k * REC, pos0 + k, 1u << k, lbits);
+            }
+            if (bmask) {
 #pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    const PairEval e = eval_pair(s, pxc[p], pyc[p], prm.alpha_min, prm.alpha_max);
-                    al[p] = e.alpha;
-                    ok[p] = !done[p] && !e.skip;
-                }
-                float wgt[NP];
-                bool any = false;
-                const int pos = (int)(b0 - start) + k + 1;
-#pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    const float Tn = T[p] * (1.f - al[p]);
-                    const bool stop = ok[p] && Tn < prm.T_min;
-                    const bool b = ok[p] && !stop;
-                    done[p] = done[p] || stop;
-                    wgt[p] = b ? al[p] * T[p] : 0.f;
-                    T[p] = b ? Tn : T[p];
-                    last[p] = b ? pos : last[p];
-                    if constexpr (CNT) blended[p] += b ? 1 : 0;
-                    any = any || b;
-                    if (SH::PIX_GROUPS) lbits[p % NL] |= (b ? 1u : 0u) << (k & 31);
-                }
-                if (!SH::PIX_GROUPS) lbits[0] |= (any ? 1u : 0u) << (k & 31);
-                if (!any) continue;
-                const float4 c = s_rgbd[k];
-#pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    const float w = wgt[p];
-                    ar[p] = fmaf(w, c.x, ar[p]);
-                    ag[p] = fmaf(w, c.y, ag[p]);
-                    ab[p] = fmaf(w, c.z, ab[p]);
-                    ad[p] = fmaf(w, c.w, ad[p]);
-                    as[p] += w;
-                }
-#pragma unroll
-                for (int q = 0; q < D4; ++q) {
-                    const float4 f = s_feat[k * D4 + q];
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        af[p][4 * q] = fmaf(wgt[p], f.x, af[p][4 * q]);
-                        af[p][4 * q + 1] = fmaf(wgt[p], f.y, af[p][4 * q + 1]);
-                        af[p][4 * q + 2] = fmaf(wgt[p], f.z, af[p][4 * q + 2]);
-                        af[p][4 * q + 3] = fmaf(wgt[p], f.w, af[p][4 * q + 3]);
-                    }
+                for (int l = 0; l < NP; ++l) {
+                    const uint32_t mine =
+                        SH::PIX_GROUPS ? lbits[l % NL] : ((SH::lanes_of_group(l) >> lane) & 1u ? lbits[0] : 0u);
+                    const uint32_t word = __reduce_or_sync(0xffffffffu, mine);
+                    if (lane == 0 && word)
+                        atomicOr(&bmask[(int64_t)SH::group(warp, l) * bm_stride + ((b0 + c0) >> 5)], word);
                 }
             }
-            if (bmask) flush(lbits, (b0 + c0) >> 5);
         }
     }
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        if (!inside[p]) continue;
-        const int64_t pix = vt.pix_off[v] + (int64_t)((int)pyc[p]) * vt.W[v] + (int)pxc[p];
-        o_rgb[pix] = ar[p] + T[p] * prm.bg[0];
-        o_rgb[P + pix] = ag[p] + T[p] * prm.bg[1];
-        o_rgb[2 * P + pix] = ab[p] + T[p] * prm.bg[2];
-        o_depth[pix] = ad[p];
-        o_sil[pix] = as[p];
-#pragma unroll
-        for (int d = 0; d < D; ++d) o_feat[d * P + pix] = af[p][d];
-        o_T[pix] = T[p];
-        o_nc[pix] = last[p];
-        if (CNT && o_nb) o_nb[pix] = blended[p];
-    }
+    px.write(vt, prm, v, tx, ty, tid, P, o_rgb, o_depth, o_sil, o_feat, o_T, o_nc, o_nb);
 }
 
 // With QUEUE, the grid is as many CTAs as fit on the GPU at once and each takes tiles, in the
@@ -265,12 +302,11 @@ __global__ void __launch_bounds__(32, fwd_group_min_blocks(D, NP)) raster_fwd_gr
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
     using SH = Shape<NP, true>;  // horizontal pixel pairs
-    constexpr int D4 = D / 4, DD = D > 0 ? D : 1;
+    constexpr int D4 = D / 4;
     constexpr int NL = SH::PIX_GROUPS ? NP : 1;  // mask bit registers per thread
     constexpr int GW = SH::WARPS;  // pixel-group blocks per tile
-    __shared__ SplatGeo s_geo[32];
-    __shared__ float4 s_rgbd[32];
-    __shared__ float4 s_feat[32 * (D4 > 0 ? D4 : 1)];
+    constexpr int REC = kRecWords<D>;
+    __shared__ float4 s_rec[32 * REC];
 
     if (binning_failed(status)) return;  // the binning overflowed or gave up: render nothing
     const int rank = blockIdx.x / GW, grp = blockIdx.x % GW;
@@ -289,32 +325,10 @@ __global__ void __launch_bounds__(32, fwd_group_min_blocks(D, NP)) raster_fwd_gr
     const float bcx = (float)(tx * kTile + bx0) + 0.5f * SH::BW, bcy = (float)(ty * kTile + by0) + 0.5f * SH::BH;
     const float hx = 0.5f * (SH::BW - 1), hy = 0.5f * (SH::BH - 1);
 
-    float pxc[NP], pyc[NP], T[NP], ar[NP], ag[NP], ab[NP], ad[NP], as[NP], af[NP][DD];
-    int last[NP], blended[NP];
-    bool inside[NP], done[NP];
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        int lx, ly;
-        SH::pixel(tid, p, lx, ly);
-        const int px = tx * kTile + lx, py = ty * kTile + ly;
-        inside[p] = px < vt.W[v] && py < vt.H[v];
-        done[p] = !inside[p];
-        pxc[p] = (float)px + 0.5f;
-        pyc[p] = (float)py + 0.5f;
-        T[p] = 1.f;
-        ar[p] = ag[p] = ab[p] = ad[p] = as[p] = 0.f;
-#pragma unroll
-        for (int d = 0; d < DD; ++d) af[p][d] = 0.f;
-        last[p] = blended[p] = 0;
-    }
-    auto all_done = [&]() {
-        bool a = true;
-#pragma unroll
-        for (int p = 0; p < NP; ++p) a = a && done[p];
-        return a;
-    };
+    BlendPixels<D, NP> px;
+    px.init(vt, prm, v, tx, ty, tid);
     for (uint32_t b0 = start & ~31u; b0 < end; b0 += 32) {
-        if (__all_sync(0xffffffffu, all_done())) break;
+        if (__all_sync(0xffffffffu, px.all_done())) break;
         // lane k stages splat b0 + k and tests whether it can reach the group's box
         bool reach = false;
         {
@@ -323,14 +337,13 @@ __global__ void __launch_bounds__(32, fwd_group_min_blocks(D, NP)) raster_fwd_gr
                 const uint32_t item = checked_item(vals[j], voff, vt.n, status);
                 const int64_t g = (int64_t)item - voff;
                 const float4 a = uvdo[item];
-                const float4 c = conic[item];
-                const SplatGeo sg = make_geo(a, uv_lo[item], c);
-                s_geo[lane] = sg;
-                reach = reaches_box(a.x, a.y, splat_extent(c, a.w, prm.alpha_min), bcx, bcy, hx, hy) &&
-                        reaches_box_exact(sg, ellipse_cull(sg, prm.alpha_min), bcx, bcy, hx, hy);
-                s_rgbd[lane] = load_rgbd(rgb, g, a.z);
+                const SplatGeo sg = make_geo(a, uv_lo[item], conic[item]);
+                float4 *rec = s_rec + lane * REC;
+                put_geo(rec, sg);
+                reach = reaches_box_exact(sg, ellipse_cull(sg, prm.alpha_min), bcx, bcy, hx, hy);
+                rec[2] = load_rgbd(rgb, g, a.z);
 #pragma unroll
-                for (int q = 0; q < D4; ++q) s_feat[lane * D4 + q] = load_feat4(feat, g * D + 4 * q);
+                for (int q = 0; q < D4; ++q) rec[3 + q] = load_feat4(feat, g * D + 4 * q);
             }
         }
         uint32_t todo = __ballot_sync(0xffffffffu, reach);
@@ -341,55 +354,8 @@ __global__ void __launch_bounds__(32, fwd_group_min_blocks(D, NP)) raster_fwd_gr
         for (int n_run = 0; todo; ++n_run) {
             const int k = __ffs(todo) - 1;
             todo &= todo - 1;
-            if ((n_run & 3) == 0 && __all_sync(0xffffffffu, all_done())) break;
-            const SplatGeo sg = s_geo[k];
-            float al[NP];
-            bool ok[NP];
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const PairEval e = eval_pair(sg, pxc[p], pyc[p], prm.alpha_min, prm.alpha_max);
-                al[p] = e.alpha;
-                ok[p] = !done[p] && !e.skip;
-            }
-            float wgt[NP];
-            bool any = false;
-            const int pos = (int)(b0 - start) + k + 1;
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const float Tn = T[p] * (1.f - al[p]);
-                const bool stop = ok[p] && Tn < prm.T_min;
-                const bool b = ok[p] && !stop;
-                done[p] = done[p] || stop;
-                wgt[p] = b ? al[p] * T[p] : 0.f;
-                T[p] = b ? Tn : T[p];
-                last[p] = b ? pos : last[p];
-                blended[p] += b ? 1 : 0;
-                any = any || b;
-                if (SH::PIX_GROUPS) lbits[p % NL] |= (b ? 1u : 0u) << k;
-            }
-            if (!SH::PIX_GROUPS) lbits[0] |= (any ? 1u : 0u) << k;
-            if (!any) continue;
-            const float4 c = s_rgbd[k];
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const float w = wgt[p];
-                ar[p] = fmaf(w, c.x, ar[p]);
-                ag[p] = fmaf(w, c.y, ag[p]);
-                ab[p] = fmaf(w, c.z, ab[p]);
-                ad[p] = fmaf(w, c.w, ad[p]);
-                as[p] += w;
-            }
-#pragma unroll
-            for (int q = 0; q < D4; ++q) {
-                const float4 f = s_feat[k * D4 + q];
-#pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    af[p][4 * q] = fmaf(wgt[p], f.x, af[p][4 * q]);
-                    af[p][4 * q + 1] = fmaf(wgt[p], f.y, af[p][4 * q + 1]);
-                    af[p][4 * q + 2] = fmaf(wgt[p], f.z, af[p][4 * q + 2]);
-                    af[p][4 * q + 3] = fmaf(wgt[p], f.w, af[p][4 * q + 3]);
-                }
-            }
+            if ((n_run & 3) == 0 && __all_sync(0xffffffffu, px.all_done())) break;
+            px.template blend<true>(prm, s_rec + k * REC, (int)(b0 - start) + k + 1, 1u << k, lbits);
         }
         if (bmask) {
             // the chunk is one mask word; words at a tile's ends are shared with the
@@ -404,31 +370,14 @@ __global__ void __launch_bounds__(32, fwd_group_min_blocks(D, NP)) raster_fwd_gr
         }
         __syncwarp();  // every lane is done with the staged chunk before the next one
     }
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        if (!inside[p]) continue;
-        const int64_t pix = vt.pix_off[v] + (int64_t)((int)pyc[p]) * vt.W[v] + (int)pxc[p];
-        o_rgb[pix] = ar[p] + T[p] * prm.bg[0];
-        o_rgb[P + pix] = ag[p] + T[p] * prm.bg[1];
-        o_rgb[2 * P + pix] = ab[p] + T[p] * prm.bg[2];
-        o_depth[pix] = ad[p];
-        o_sil[pix] = as[p];
-#pragma unroll
-        for (int d = 0; d < D; ++d) o_feat[d * P + pix] = af[p][d];
-        o_T[pix] = T[p];
-        o_nc[pix] = last[p];
-        if (o_nb) o_nb[pix] = blended[p];
-    }
+    px.write(vt, prm, v, tx, ty, tid, P, o_rgb, o_depth, o_sil, o_feat, o_T, o_nc, o_nb);
 }
 
 // One batch slot of the ring forward: B staged splat records.
 template <int D, int B>
 struct RingSlot {
-    SplatGeo geo[B];
-    float2 ext[B];
+    float4 rec[B * kRecWords<D>];
     float4 cull[B];
-    float4 rgbd[B];
-    float4 feat[B * (D / 4 > 0 ? D / 4 : 1)];
 };
 
 // The per-tile forward with its splats staged into a ring of NBUF batch slots of B records:
@@ -453,7 +402,7 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
     using SH = Shape<NP, true>;  // horizontal pixel pairs
     constexpr int NT = SH::THREADS, NW = SH::WARPS;
     constexpr int NL = SH::PIX_GROUPS ? NP : 1;
-    constexpr int D4 = D / 4, DD = D > 0 ? D : 1;
+    constexpr int D4 = D / 4;
     constexpr int QB = B / NW;  // records a warp stages per batch
     static_assert(B % 32 == 0 && QB <= 32 && NBUF >= 2, "ring shape");
     __shared__ RingSlot<D, B> s_slot[NBUF];
@@ -492,14 +441,13 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
                 const uint32_t item = checked_item(vals[jj], voff, vt.n, status);
                 const int64_t g = (int64_t)item - voff;
                 const float4 a = uvdo[item];
-                const float4 c = conic[item];
-                const SplatGeo sg = make_geo(a, uv_lo[item], c);
-                S.geo[k] = sg;
-                S.ext[k] = splat_extent(c, a.w, prm.alpha_min);
+                const SplatGeo sg = make_geo(a, uv_lo[item], conic[item]);
+                float4 *rec = S.rec + k * kRecWords<D>;
+                put_geo(rec, sg);
                 S.cull[k] = ellipse_cull(sg, prm.alpha_min);
-                S.rgbd[k] = load_rgbd(rgb, g, a.z);
+                rec[2] = load_rgbd(rgb, g, a.z);
 #pragma unroll
-                for (int q = 0; q < D4; ++q) S.feat[k * D4 + q] = load_feat4(feat, g * D + 4 * q);
+                for (int q = 0; q < D4; ++q) rec[3 + q] = load_feat4(feat, g * D + 4 * q);
             }
         }
         if (lane == 0) s_stop[j % NBUF][warp] = *(volatile int *)&s_done == NW;
@@ -510,30 +458,8 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
     SH::warp_origin(warp, bx0, by0);
     const float bcx = (float)(tx * kTile + bx0) + 0.5f * SH::BW, bcy = (float)(ty * kTile + by0) + 0.5f * SH::BH;
     const float hx = 0.5f * (SH::BW - 1), hy = 0.5f * (SH::BH - 1);
-    float pxc[NP], pyc[NP], T[NP], ar[NP], ag[NP], ab[NP], ad[NP], as[NP], af[NP][DD];
-    int last[NP], blended[NP];
-    bool inside[NP], done[NP];
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        int lx, ly;
-        SH::pixel(tid, p, lx, ly);
-        const int px = tx * kTile + lx, py = ty * kTile + ly;
-        inside[p] = px < vt.W[v] && py < vt.H[v];
-        done[p] = !inside[p];
-        pxc[p] = (float)px + 0.5f;
-        pyc[p] = (float)py + 0.5f;
-        T[p] = 1.f;
-        ar[p] = ag[p] = ab[p] = ad[p] = as[p] = 0.f;
-#pragma unroll
-        for (int d = 0; d < DD; ++d) af[p][d] = 0.f;
-        last[p] = blended[p] = 0;
-    }
-    auto all_done = [&]() {
-        bool a = true;
-#pragma unroll
-        for (int p = 0; p < NP; ++p) a = a && done[p];
-        return a;
-    };
+    BlendPixels<D, NP> px;
+    px.init(vt, prm, v, tx, ty, tid);
     auto flush = [&](const uint32_t (&lbits)[NL], uint32_t word_idx) {
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
@@ -566,7 +492,7 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
         if (stop) break;  // the same batch for every warp: every pixel of the tile is done
         const RingSlot<D, B> &S = s_slot[slot];
         const uint32_t b0 = first + (uint32_t)i * B;
-        if (!__all_sync(0xffffffffu, all_done())) {
+        if (!__all_sync(0xffffffffu, px.all_done())) {
             const int k_lo = b0 < start ? (int)(start - b0) : 0;
             const int nb = min((uint32_t)B, end - b0);
             bool finished = false;
@@ -577,68 +503,21 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
                 const int kl = c0 + lane;
                 bool reach = false;
                 if (kl >= k_lo && kl < nb) {
-                    const SplatGeo sg = S.geo[kl];
-                    reach = reaches_box(sg.u, sg.v, S.ext[kl], bcx, bcy, hx, hy) &&
-                            reaches_box_exact(sg, S.cull[kl], bcx, bcy, hx, hy);
+                    const SplatGeo sg = geo_of(S.rec + kl * kRecWords<D>);
+                    reach = reaches_box_exact(sg, S.cull[kl], bcx, bcy, hx, hy);
                 }
                 uint32_t todo = __ballot_sync(0xffffffffu, reach);
                 for (int n_run = 0; todo; ++n_run) {
                     const int k = c0 + __ffs(todo) - 1;
                     todo &= todo - 1;
-                    if ((n_run & 3) == 0 && __all_sync(0xffffffffu, all_done())) { finished = true; break; }
-                    const SplatGeo s = S.geo[k];
-                    float al[NP];
-                    bool okp[NP];
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        const PairEval e = eval_pair(s, pxc[p], pyc[p], prm.alpha_min, prm.alpha_max);
-                        al[p] = e.alpha;
-                        okp[p] = !done[p] && !e.skip;
-                    }
-                    float wgt[NP];
-                    bool any = false;
-                    const int pos = (int)(b0 - start) + k + 1;
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        const float Tn = T[p] * (1.f - al[p]);
-                        const bool stp = okp[p] && Tn < prm.T_min;
-                        const bool b = okp[p] && !stp;
-                        done[p] = done[p] || stp;
-                        wgt[p] = b ? al[p] * T[p] : 0.f;
-                        T[p] = b ? Tn : T[p];
-                        last[p] = b ? pos : last[p];
-                        blended[p] += b ? 1 : 0;
-                        any = any || b;
-                        if (SH::PIX_GROUPS) lbits[p % NL] |= (b ? 1u : 0u) << (k & 31);
-                    }
-                    if (!SH::PIX_GROUPS) lbits[0] |= (any ? 1u : 0u) << (k & 31);
-                    if (!any) continue;
-                    const float4 c = S.rgbd[k];
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        const float w = wgt[p];
-                        ar[p] = fmaf(w, c.x, ar[p]);
-                        ag[p] = fmaf(w, c.y, ag[p]);
-                        ab[p] = fmaf(w, c.z, ab[p]);
-                        ad[p] = fmaf(w, c.w, ad[p]);
-                        as[p] += w;
-                    }
-#pragma unroll
-                    for (int q = 0; q < D4; ++q) {
-                        const float4 f = S.feat[k * D4 + q];
-#pragma unroll
-                        for (int p = 0; p < NP; ++p) {
-                            af[p][4 * q] = fmaf(wgt[p], f.x, af[p][4 * q]);
-                            af[p][4 * q + 1] = fmaf(wgt[p], f.y, af[p][4 * q + 1]);
-                            af[p][4 * q + 2] = fmaf(wgt[p], f.z, af[p][4 * q + 2]);
-                            af[p][4 * q + 3] = fmaf(wgt[p], f.w, af[p][4 * q + 3]);
-                        }
-                    }
+                    if ((n_run & 3) == 0 && __all_sync(0xffffffffu, px.all_done())) { finished = true; break; }
+                    px.template blend<true>(prm, S.rec + k * kRecWords<D>, (int)(b0 - start) + k + 1, 1u << (k & 31),
+                                            lbits);
                 }
                 if (bmask) flush(lbits, (b0 + c0) >> 5);
             }
         }
-        if (!counted && __all_sync(0xffffffffu, all_done())) {
+        if (!counted && __all_sync(0xffffffffu, px.all_done())) {
             counted = true;
             if (lane == 0) atomicAdd(&s_done, 1);
         }
@@ -658,21 +537,7 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
         set_status(status, GS_ERR_TIMEOUT);
         return;  // this warp's pixels stay unwritten; the status word says so
     }
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        if (!inside[p]) continue;
-        const int64_t pix = vt.pix_off[v] + (int64_t)((int)pyc[p]) * vt.W[v] + (int)pxc[p];
-        o_rgb[pix] = ar[p] + T[p] * prm.bg[0];
-        o_rgb[P + pix] = ag[p] + T[p] * prm.bg[1];
-        o_rgb[2 * P + pix] = ab[p] + T[p] * prm.bg[2];
-        o_depth[pix] = ad[p];
-        o_sil[pix] = as[p];
-#pragma unroll
-        for (int d = 0; d < D; ++d) o_feat[d * P + pix] = af[p][d];
-        o_T[pix] = T[p];
-        o_nc[pix] = last[p];
-        if (o_nb) o_nb[pix] = blended[p];
-    }
+    px.write(vt, prm, v, tx, ty, tid, P, o_rgb, o_depth, o_sil, o_feat, o_T, o_nc, o_nb);
 }
 
 template <int D, int NP, typename RT, typename FT>

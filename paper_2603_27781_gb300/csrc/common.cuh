@@ -14,6 +14,7 @@
 namespace gs {
 
 constexpr int kMaxViews = 64;
+constexpr int kSMs = 152;  // of a GB300: rules that weigh work against the chip's size
 constexpr int kTile = 16;
 constexpr int kTilePix = kTile * kTile;  // one thread per pixel, 8 warps per tile
 constexpr float kLog2e = 1.4426950408889634f;

@@ -34,9 +34,13 @@ __device__ __forceinline__ void put_geo(float4 *rec, const SplatGeo &s) {
     rec[1] = make_float4(s.qa, s.qb, s.qc, s.o);
 }
 
-// The pixels of one thread while they are blended: position, transmittance, the alpha below which
-// a splat is skipped (alpha_min, and infinity once the pixel is done or lies outside the image) and
-// the blended sums.  The sums are kept as packed pairs of channels ((r, g), (b, depth), the
+// Splats evaluated together: four with two pixels per thread (forward of 1M Gaussians at 1200x680, D =
+// 16: 0.231 ms, against 0.233 with two and 0.254 with one; D = 32 at 640x480: 0.163, 0.175, 0.192),
+// two with one pixel, whose kernels have half the registers (D = 8: 0.075, 0.077 with four or one).
+constexpr int walk_splats(int NP) { return NP == 2 ? 4 : NP == 1 ? 2 : 1; }
+
+// The pixels of one thread while they are blended: position, transmittance, whether the pixel is done
+// (stopped, or outside the image) and the blended sums.  The sums are kept as packed pairs of channels ((r, g), (b, depth), the
 // features), which match the 16-byte words of the staged records, so a splat costs (4 + D) / 2
 // packed multiply-adds per pixel instead of 4 + D scalar ones, with the same rounding.
 //
@@ -55,7 +59,9 @@ struct BlendPixels {
     using SH = Shape<NP, true>;  // horizontal pixel pairs
     static constexpr int NL = SH::PIX_GROUPS ? NP : 1;  // mask bit registers per thread
     static constexpr int D4 = D / 4, F4 = D4 > 0 ? D4 : 1;
-    float pxc[NP], pyc[NP], T[NP], lim[NP], as[NP];
+    static constexpr int kWalk = walk_splats(NP);
+    float pxc[NP], pyc[NP], T[NP], as[NP];
+    bool done[NP];
     float2 acc[NP][2], af[NP][2 * F4];
     int last[NP], blended[NP];
 
@@ -68,7 +74,7 @@ struct BlendPixels {
             pxc[p] = (float)px + 0.5f;
             pyc[p] = (float)py + 0.5f;
             T[p] = 1.f;
-            lim[p] = px < vt.W[v] && py < vt.H[v] ? prm.alpha_min : INFINITY;
+            done[p] = !(px < vt.W[v] && py < vt.H[v]);
             as[p] = 0.f;
             acc[p][0] = acc[p][1] = make_float2(0.f, 0.f);
 #pragma unroll
@@ -79,23 +85,29 @@ struct BlendPixels {
     __device__ __forceinline__ bool all_done() const {
         bool a = true;
 #pragma unroll
-        for (int p = 0; p < NP; ++p) a = a && lim[p] == INFINITY;
+        for (int p = 0; p < NP; ++p) a = a && done[p];
         return a;
     }
-    // Blends one staged splat (its record, list position pos, mask bit `bit`) into the thread's pixels.
-    template <bool CNT>
-    __device__ __forceinline__ void blend(const Params &prm, const float4 *rec, int pos, uint32_t bit,
-                                          uint32_t (&lbits)[NL]) {
+    // The splat's alpha at each of the thread's pixels, which does not depend on what is in front.
+    __device__ __forceinline__ void evaluate(const Params &prm, const float4 *rec, PairEval (&e)[NP]) const {
         const SplatGeo s = geo_of(rec);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) e[p] = eval_pair(s, pxc[p], pyc[p], prm.alpha_min, prm.alpha_max);
+    }
+    // Blends one evaluated splat (its record, list position pos, mask bit `bit`) into the thread's pixels.
+    template <bool CNT>
+    __device__ __forceinline__ void blend(const Params &prm, const PairEval (&ev)[NP], const float4 *rec, int pos,
+                                          uint32_t bit, uint32_t (&lbits)[NL]) {
         float wgt[NP];
         bool any = false;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            const PairEval e = eval_pair(s, pxc[p], pyc[p], lim[p], prm.alpha_max);
+            const PairEval &e = ev[p];
             const float Tn = T[p] * (1.f - e.alpha);
-            const bool stop = !e.skip && Tn < prm.T_min;
-            const bool b = !e.skip && !stop;
-            lim[p] = stop ? INFINITY : lim[p];
+            const bool ok = !e.skip && !done[p];
+            const bool stop = ok && Tn < prm.T_min;
+            const bool b = ok && !stop;
+            done[p] = done[p] || stop;
             wgt[p] = b ? e.alpha * T[p] : 0.f;
             T[p] = b ? Tn : T[p];
             last[p] = b ? pos : last[p];
@@ -123,6 +135,33 @@ struct BlendPixels {
                 af[p][2 * q + 1] = fma2(w, make_float2(f.z, f.w), af[p][2 * q + 1]);
             }
         }
+    }
+    // Walks the splats of `todo` (bit k: record k of the chunk, list position pos0 + k) front to back
+    // and sets the bits of those blended; true once all of the warp's pixels are done.  kWalk splats
+    // are evaluated together before they are blended in order, so their loads and exponentials
+    // overlap; whether the warp is done is looked at every fourth splat (a later exit only runs
+    // splats whose pairs blend nothing).
+    template <bool CNT>
+    __device__ __forceinline__ bool walk(const Params &prm, const float4 *chunk, uint32_t todo, int pos0,
+                                         uint32_t (&lbits)[NL]) {
+        constexpr int REC = kRecWords<D>;
+        for (int run = 0; todo; run += kWalk) {
+            if ((run & 3) == 0 && __all_sync(0xffffffffu, all_done())) return true;
+            int k[kWalk];
+            bool has[kWalk];
+            PairEval e[kWalk][NP];
+#pragma unroll
+            for (int u = 0; u < kWalk; ++u) {
+                has[u] = todo != 0u;  // warp-uniform
+                k[u] = has[u] ? __ffs(todo) - 1 : k[u > 0 ? u - 1 : 0];
+                todo &= todo - 1u;
+                evaluate(prm, chunk + k[u] * REC, e[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < kWalk; ++u)
+                if (u == 0 || has[u]) blend<CNT>(prm, e[u], chunk + k[u] * REC, pos0 + k[u], 1u << k[u], lbits);
+        }
+        return false;
     }
     __device__ __forceinline__ void write(const ViewTable &vt, const Params &prm, int v, int tx, int ty, int tid, int64_t P,
                                           float *o_rgb, float *o_depth, float *o_sil, float *o_feat, float *o_T,
@@ -209,7 +248,7 @@ __device__ __forceinline__ void fwd_tile(
             const float4 *chunk = s_rec + c0 * REC;
             const bool reach = j >= start && j < end &&
                                reaches_box_exact(geo_of(chunk + lane * REC), s_cull[c0 + lane], bcx, bcy, hx, hy);
-            uint32_t todo = __ballot_sync(0xffffffffu, reach);
+            const uint32_t todo = __ballot_sync(0xffffffffu, reach);
             if (todo == 0u) continue;
             // blend-mask bits: batches start on 32-instance boundaries, so each 32-splat chunk is one
             // word of the mask; a lane ORs "my pixel(s) of group j blended splat k" into a register
@@ -219,14 +258,7 @@ __device__ __forceinline__ void fwd_tile(
 #pragma unroll
             for (int l = 0; l < NL; ++l) lbits[l] = 0u;
             const int pos0 = (int)(b0 + c0 - start) + 1;
-            for (int n_run = 0; todo; ++n_run) {
-                const int k = __ffs(todo) - 1;
-                todo &= todo - 1;
-                // every 4th splat walked: are all of the warp's pixels done? (a later exit only
-                // runs splats whose pairs blend nothing)
-                if ((n_run & 3) == 0 && __all_sync(0xffffffffu, px.all_done())) { finished = true; break; }
-                px.template blend<CNT>(prm, chunk + k * REC, pos0 + k, 1u << k, lbits);
-            }
+            finished = px.template walk<CNT>(prm, chunk, todo, pos0, lbits);
             if (bmask) {
 #pragma unroll
                 for (int l = 0; l < NP; ++l) {
@@ -346,17 +378,12 @@ __global__ void __launch_bounds__(32, fwd_group_min_blocks(D, NP)) raster_fwd_gr
                 for (int q = 0; q < D4; ++q) rec[3 + q] = load_feat4(feat, g * D + 4 * q);
             }
         }
-        uint32_t todo = __ballot_sync(0xffffffffu, reach);
+        const uint32_t todo = __ballot_sync(0xffffffffu, reach);
         __syncwarp();
         uint32_t lbits[NL];
 #pragma unroll
         for (int j = 0; j < NL; ++j) lbits[j] = 0u;
-        for (int n_run = 0; todo; ++n_run) {
-            const int k = __ffs(todo) - 1;
-            todo &= todo - 1;
-            if ((n_run & 3) == 0 && __all_sync(0xffffffffu, px.all_done())) break;
-            px.template blend<true>(prm, s_rec + k * REC, (int)(b0 - start) + k + 1, 1u << k, lbits);
-        }
+        px.template walk<true>(prm, s_rec, todo, (int)(b0 - start) + 1, lbits);
         if (bmask) {
             // the chunk is one mask word; words at a tile's ends are shared with the
             // neighbouring tile's blocks, hence the atomic OR
@@ -506,14 +533,8 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
                     const SplatGeo sg = geo_of(S.rec + kl * kRecWords<D>);
                     reach = reaches_box_exact(sg, S.cull[kl], bcx, bcy, hx, hy);
                 }
-                uint32_t todo = __ballot_sync(0xffffffffu, reach);
-                for (int n_run = 0; todo; ++n_run) {
-                    const int k = c0 + __ffs(todo) - 1;
-                    todo &= todo - 1;
-                    if ((n_run & 3) == 0 && __all_sync(0xffffffffu, px.all_done())) { finished = true; break; }
-                    px.template blend<true>(prm, S.rec + k * kRecWords<D>, (int)(b0 - start) + k + 1, 1u << (k & 31),
-                                            lbits);
-                }
+                const uint32_t todo = __ballot_sync(0xffffffffu, reach);
+                finished = px.template walk<true>(prm, S.rec + c0 * kRecWords<D>, todo, (int)(b0 - start) + c0 + 1, lbits);
                 if (bmask) flush(lbits, (b0 + c0) >> 5);
             }
         }
@@ -651,7 +672,16 @@ extern "C" gs_status gs_render_fwd(const gs_gaussians *g, const gs_projected *pr
             out->blend_mask, 0, sizeof(uint32_t) * kGroups * (size_t)(bins->capacity / 32 + 1), st));
         if (s) return s;
     }
-    const int np = prm.fwd_np ? prm.fwd_np : default_fwd_np(g->feat_dim);
+    int np = prm.fwd_np ? prm.fwd_np : default_fwd_np(g->feat_dim);
+    // The default at D = 16 and 32 is two pixels per thread, and one where the image has too few tiles for
+    // that: up to one wave of the two-pixel CTAs at D = 16 (six per SM) and two at D = 32 (four per SM) twice
+    // as many warps hide more latency.  Measured, one against two pixels per thread: D = 16: 0.023 / 0.025
+    // ms at 160x120, 0.055 / 0.059 at 320x240, 0.075 / 0.081 at 480x360, but 0.146 / 0.135 (scan) at 640x480
+    // and 0.262 / 0.231 at 1200x680; D = 32: 0.053 / 0.063 at 320x240, 0.148 / 0.163 at 640x480, but 0.114 /
+    // 0.109 at 811x607.  The images do not depend on it.
+    if (!prm.fwd_np && g->feat_dim >= 16 && prm.fwd_blocks == GS_BWD_BLOCKS_DEFAULT && prm.fwd_batch == kBatch &&
+        vt.tile_off[n_views] <= kSMs * (g->feat_dim == 16 ? 6 : 8))
+        np = 1;
     prm.fwd_group = prm.fwd_blocks == GS_BWD_BLOCKS_GROUP;
     prm.fwd_queue = prm.fwd_blocks == GS_BLOCKS_QUEUE;
     prm.fwd_ring = prm.fwd_blocks == GS_BLOCKS_RING;

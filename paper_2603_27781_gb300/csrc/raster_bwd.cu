@@ -107,8 +107,20 @@ extern "C" gs_status gs_render_bwd(const gs_gaussians *g, const gs_projected *pr
     Params pr = prm;
     pr.bwd_warp = prm.bwd_blocks == GS_BWD_BLOCKS_GROUP || (prm.bwd_blocks == GS_BWD_BLOCKS_DEFAULT && group_ok);
     if (factored && !pr.bwd_warp) return GS_ERR_UNSUPPORTED;  // the tile kernel takes the features' gradient
-    // default pixels per thread: 2 for the per-group form at D = 16 (8x8 blocks), else 1
-    const int np = prm.bwd_np ? prm.bwd_np : (pr.bwd_warp ? (D == 16 ? 2 : 1) : default_bwd_np(D));
+    // Default pixels per thread of the per-group form: two (8x8 blocks, four per tile, whose lanes share each
+    // splat's loads and shuffles over two pixels), and one (twice as many warps) where the image has too
+    // few blocks to hide latency with: below 7 two-pixel blocks per SM in map mode with the factored form,
+    // 32 (D = 16) or 20 (D = 32) otherwise, where the two-pixel kernels hold fewer warps.  Measured in ms,
+    // one against two pixels per thread:
+    //   map, factored: 0.068 / 0.096 at 64x48, 0.022 / 0.028 at 160x120, 0.070 / 0.066 at 320x240,
+    //     0.528 / 0.392 at 1200x680; D = 32: 0.279 / 0.207 at 640x480
+    //   map, features: 0.060 / 0.070 at 640x480, 0.180 / 0.164 at 811x607, 0.533 / 0.466 at 1200x680;
+    //     D = 32: 0.121 / 0.129 at 480x360, 0.373 / 0.309 at 640x480
+    //   pose: 0.150 / 0.166 at 640x480, 0.251 / 0.243 at 1200x680; D = 32: 0.191 / 0.150 at 640x480
+    const int per_sm = map && factored ? 7 : D == 16 ? 32 : 20;
+    const int np = prm.bwd_np ? prm.bwd_np
+                   : !pr.bwd_warp ? default_bwd_np(D)
+                                  : 4 * (int64_t)vt.tile_off[n_views] < (int64_t)kSMs * per_sm ? 1 : 2;
     const bool half = g->rgb_dtype == GS_F16;
     return map ? dispatch_bwd_map(D, np, half, vt, pr, A, st) : dispatch_bwd_pose(D, np, half, vt, pr, A, st);
 }

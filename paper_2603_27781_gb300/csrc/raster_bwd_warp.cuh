@@ -13,20 +13,25 @@
 // per-pixel recurrence on them.  Nothing waits on another warp, and a finished
 // group frees its resources at once.
 //
-// Map mode defers every per-splat sum.  While it walks a stage of splats, each
-// pixel only records, per splat, its weight w = alpha T (the factor of the depth,
-// colour and feature gradients) and dpow = o G dL/dalpha (zero where alpha is
-// clamped), the factor of every geometric gradient: with (lx, ly) the pixel centre
-// relative to the block centre and (cx, cy) the splat centre, dx = lx - cx, so the
-// centre and conic gradients need only the moments of dpow
-//   S1, Sx, Sy, Sxx, Sxy, Syy = sum over pixels of dpow (1, lx, ly, lx^2, lx ly, ly^2),
-// expanded about the splat centre afterwards (sum dpow dx = Sx - cx S1, and so on),
-// and the opacity gradient is S1 / o.  After the stage, lanes (pixel column, slot
-// pair) contract the slots with the block's per-pixel terms (weights against the
-// gradients of depth, colour and features; dpow against the row coordinates) down
-// their column in FP32 FMAs, the eight columns are combined by one transpose
-// reduction per stage, and each slot's sums go out as 16-byte L2 reductions.  No
-// warp reduction runs per splat.
+// Every per-splat sum is deferred.  While it walks a stage of splats, each pixel only records, per
+// splat, its weight w = alpha T (the factor of the depth, colour and feature gradients; in pose mode w
+// times the pixel's depth gradient) and dpow = o G dL/dalpha (zero where alpha is clamped), the factor
+// of every geometric gradient: with (dx, dy) the pixel centre from the splat centre, the centre and
+// conic gradients need only the moments
+//   S1, Sx, Sy, Sxx, Sxy, Syy = sum over pixels of dpow (1, dx, dy, dx^2, dx dy, dy^2),
+// and the opacity gradient is S1 / o.  After the stage, lanes (pixel column, slot pair) contract the
+// slots with the block's per-pixel terms (weights against the gradients of depth, colour and features;
+// dpow against the row's dy, the column's dx scaling the column sums afterwards) in packed FP32
+// multiply-adds, the eight columns are combined by one transpose reduction per stage, and each slot's
+// sums go out as 16-byte L2 reductions.  No warp reduction runs per splat.
+//
+// What bounds it: the shared-memory pipe (every 16-byte read returns 512 bytes to a warp, four cycles,
+// broadcast or not; about 57 cycles per splat and block at D = 16 with two pixels per thread) and
+// instruction issue, both near 70 %.  Packed multiply-adds for g.x, the contraction, z = W f and W^T z,
+// weight and dpow as one 8-byte pair, moments about the splat centre (no expansion afterwards, nothing
+// cancels) and a first reduction level without selects took the map mode from 0.417 to 0.391 ms (1M
+// Gaussians, D = 16, 1200x680) and 0.217 to 0.207 (1M, D = 32, 640x480), and the pose mode, which before
+// reduced six values over the warp for every splat, from 0.355 to 0.241 ms (300k scanned Gaussians).
 //
 // Factored feature gradients.  When the image gradient of the features comes from
 // a linear decoder (Eq. 8 read as a 1x1 convolution), g_feat = W^T e with e the
@@ -44,46 +49,52 @@ namespace gs {
 // gradients (zero beyond K).
 constexpr int kFactorK = 8;
 
-// Map-mode layout: SL slots (splats staged and contracted together); in the contraction lane
-// (column c, slot group j) sums the NWT weighted terms and the dpow column sums of SPL slots over
-// the ROWS pixels of column c, and the eight columns are then added by shuffles.  In the epilogue
-// LPS = 32 / SL lanes serve each slot.
-template <int D, int NP, int KF, int SL>
-struct WarpMapLayout {
+// Layout of the deferred sums: SL slots (splats staged and contracted together).  In the contraction
+// lane (column c, slot group jg) sums, for the SPL slots of group jg, the NWT weighted terms (map mode)
+// and the moments of dpow over the ROWS pixels of column c; the eight columns are then added by
+// shuffles.  In the epilogue LPS = 32 / SL lanes serve each slot.
+template <int D, int NP, bool MAP, int KF, int SL>
+struct WarpLayout {
     static constexpr int F = KF ? KF : D;
     static constexpr int PXW = 32 * NP;         // pixels of the block, 8 wide
     static constexpr int ROWS = PXW / 8;
     static constexpr int LPS = 32 / SL;
     static constexpr int SPL = SL / 4;          // slots per lane in the contraction
-    static constexpr int NWT = 4 + F;           // weighted terms: depth, r, g, b, F
+    static constexpr int NWT = MAP ? 4 + F : 0; // weighted terms: depth, r, g, b, F
     static constexpr int GROW = NWT;            // a pixel's row of weighted terms
-    static constexpr int NSV = NWT + 6;         // a slot's sums: the terms and six moments
+    // a slot's sums: the terms, then S1, Sx, Sy, Sxx, Sxy, Syy (map mode), or Sx, Sy, Sxx, Sxy, Syy and
+    // the depth gradient (pose mode)
+    static constexpr int NSV = NWT + 6;
     // The contraction runs in up to four chunks of terms so that a lane's running sums fit in
     // its registers (at most 2 CAPS values): the first chunk [0, T1) carries the moments,
     // then [T1, T2), [T2, T3) and [T3, NWT).
-    static constexpr int CAPS = NP == 1 ? 12 : 28;
+    static constexpr int CAPS = NP == 1 ? 12 : KF ? 28 : 18;
     static constexpr int TC = CAPS / 4 * 4;
     static constexpr int T1 = NWT < (CAPS - 6) / 4 * 4 ? NWT : (CAPS - 6) / 4 * 4;
     static constexpr int T2 = NWT < T1 + TC ? NWT : T1 + TC;
     static constexpr int T3 = NWT < T2 + TC ? NWT : T2 + TC;
     static_assert(NWT <= T3 + TC, "four chunks cover the terms");
-    static constexpr int WROW = PXW + 4;        // a slot's row of per-pixel values (padded against bank conflicts)
-    static_assert(NWT % 4 == 0 && SL == 8 && D % (4 * LPS) == 0, "16-byte rows; lanes divide the work");
+    // a slot's row of per-pixel pairs: 8 words beyond a multiple of 32, which spreads the contraction's
+    // reads (two slots a group, taken in opposite order by even and odd columns) over all banks
+    static constexpr int WROW = PXW + 4;
+    static_assert(NWT % 4 == 0 && SL % 8 == 0 && SPL % 2 == 0 && (!MAP || D % (4 * LPS) == 0),
+                  "16-byte rows; lanes divide the work");
 };
 
 template <int V> struct IntC { static constexpr int value = V; };
 
-// Slots per stage in map mode: 8 (four lanes per slot) keeps the per-slot arrays small
-// enough for more resident blocks; pose mode stages 16.
-constexpr int kMapSlots = 8;
-constexpr int kPoseStage = 16;
+// Slots per stage: 8 (four lanes per slot) keeps the per-slot arrays small enough for more
+// resident blocks (pose mode, 300k scanned Gaussians at 1200x680: 0.241 ms, 0.265 with 16).
+constexpr int kSlots = 8;
 
-// Resident blocks per SM the register allocation must allow: 24 with one pixel per thread
-// (80 registers), 16 with two (128), except where 16 would spill at D = 32: the map mode with
-// the features themselves (whose 19.5 KB of shared memory allows 11 blocks anyway) and the
-// pose mode with the factored form.
+// Resident blocks per SM the register allocation must allow: 16 with two pixels per thread (128
+// registers), except the map mode with the features themselves at D = 32 (whose 19 KB of shared memory
+// allows 11 anyway) and the pose mode with the factored form at D = 32 (12); with one pixel per thread 24 (80
+// registers) in pose mode and 20 or 18 in map mode, where 24 would spill (features themselves, 100k
+// Gaussians at 640x480, D = 16: 0.060 against 0.077 ms).
 template <int D, int NP, bool MAP, int KF> constexpr int warp_bwd_min_blocks() {
-    return NP == 1 ? 24 : (D == 32 && (MAP ? KF == 0 : KF > 0)) ? (MAP ? 11 : 12) : 16;
+    if (NP == 1) return !MAP ? 24 : (D == 32 && KF == 0) ? 18 : 20;
+    return (D == 32 && (MAP ? KF == 0 : KF > 0)) ? (MAP ? 11 : 12) : 16;
 }
 
 template <int D, int NP, bool MAP, int KF, typename RT, typename FT>
@@ -92,12 +103,12 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
     using SH = Shape<NP>;
-    using WL = WarpMapLayout<D, NP, KF, kMapSlots>;
+    constexpr int STAGE = kSlots;
+    using WL = WarpLayout<D, NP, MAP, KF, STAGE>;
     constexpr int F = WL::F;
     constexpr int F4 = F / 4;
-    constexpr int NCH = 5 + F;            // r, g, b, depth, sil, then F
+    constexpr int NC2 = 2 + F / 2;        // channel pairs: (r, g), (b, depth), then F
     constexpr int GW = SH::WARPS;         // pixel-group blocks per tile
-    constexpr int STAGE = MAP ? kMapSlots : kPoseStage;
     constexpr int PARTS = 32 / STAGE;     // lanes per staged splat
     static_assert(F % 4 == 0 && (KF == 0 || KF % PARTS == 0), "staged values in float4 / lane parts");
     __shared__ SplatGeo s_geo[STAGE];
@@ -106,10 +117,10 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
     __shared__ uint32_t s_item[STAGE];
     __shared__ int s_pos[STAGE];
     __shared__ uint32_t s_list[64];
-    __shared__ __align__(16) float s_w[MAP ? STAGE * WL::WROW : 4];   // [slot][pixel] alpha T
-    __shared__ __align__(16) float s_p[MAP ? STAGE * WL::WROW : 4];   // [slot][pixel] dpow
+    __shared__ float2 s_ctr[STAGE];                                   // splat centre from the block's
+    __shared__ float2 s_wp[STAGE * WL::WROW];                         // [slot][pixel] weight, dpow
     __shared__ __align__(16) float s_g[MAP ? WL::PXW * WL::GROW : 4]; // [pixel][term] gradients
-    __shared__ float s_t[MAP ? STAGE * WL::NSV : 4];                  // [slot][sum] sums
+    __shared__ float s_t[STAGE * WL::NSV];                            // [slot][sum] sums
     // W, K x D (rows >= K zero), rows padded by 4 so that the four lane parts, which read rows
     // k = part (K / 4) + kk, fall in different banks
     constexpr int BROW = D + 4;
@@ -154,7 +165,8 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
             s_basis[(i / D) * BROW + i % D] = i < A.feat_rank * D ? A.feat_basis[i] : 0.f;
     }
 
-    float gch[NP][NCH], T[NP], gS[NP], pxc[NP], pyc[NP];
+    float2 gch[NP][NC2];  // gradients of the channel pairs
+    float gsil[NP], T[NP], gS[NP], pxc[NP], pyc[NP];
     int last[NP];
     int my_max = 0;
 #pragma unroll
@@ -167,25 +179,25 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
         T[p] = 1.f;
         last[p] = 0;
 #pragma unroll
-        for (int c = 0; c < NCH; ++c) gch[p][c] = 0.f;
+        for (int c = 0; c < NC2; ++c) gch[p][c] = make_float2(0.f, 0.f);
+        gsil[p] = 0.f;
         if (px < vt.W[v] && py < vt.H[v]) {
             const int64_t pix = vt.pix_off[v] + (int64_t)py * vt.W[v] + px;
             T[p] = A.T_final[pix];
             last[p] = A.n_contrib[pix];
-            gch[p][0] = A.g_rgb[pix];
-            gch[p][1] = A.g_rgb[P + pix];
-            gch[p][2] = A.g_rgb[2 * P + pix];
-            gch[p][3] = A.g_depth[pix];
-            gch[p][4] = A.g_sil ? A.g_sil[pix] : 0.f;
-            if constexpr (KF > 0) {
+            gch[p][0] = make_float2(A.g_rgb[pix], A.g_rgb[P + pix]);
+            gch[p][1] = make_float2(A.g_rgb[2 * P + pix], A.g_depth[pix]);
+            gsil[p] = A.g_sil ? A.g_sil[pix] : 0.f;
 #pragma unroll
-                for (int k = 0; k < KF; ++k) gch[p][5 + k] = k < A.feat_rank ? A.feat_coef[k * P + pix] : 0.f;
-            } else {
-#pragma unroll
-                for (int d = 0; d < D; ++d) gch[p][5 + d] = A.g_feat[d * P + pix];
+            for (int c = 0; c < F / 2; ++c) {
+                if constexpr (KF > 0)
+                    gch[p][2 + c] = make_float2(2 * c < A.feat_rank ? A.feat_coef[2 * c * P + pix] : 0.f,
+                                                2 * c + 1 < A.feat_rank ? A.feat_coef[(2 * c + 1) * P + pix] : 0.f);
+                else
+                    gch[p][2 + c] = make_float2(A.g_feat[2 * c * P + pix], A.g_feat[(2 * c + 1) * P + pix]);
             }
         }
-        gS[p] = gch[p][0] * prm.bg[0] + gch[p][1] * prm.bg[1] + gch[p][2] * prm.bg[2];
+        gS[p] = gch[p][0].x * prm.bg[0] + gch[p][0].y * prm.bg[1] + gch[p][1].x * prm.bg[2];
         my_max = max(my_max, last[p]);
     }
     const int wmax = checked_last(start, A.ranges, gt, __reduce_max_sync(0xffffffffu, my_max), A.capacity, A.status);
@@ -194,94 +206,115 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
         // pixel q = p * 32 + lane of the block: its weighted terms (depth, r, g, b, F), part by part
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            float term[WL::NWT];
-            term[0] = gch[p][3];
-            term[1] = gch[p][0];
-            term[2] = gch[p][1];
-            term[3] = gch[p][2];
-#pragma unroll
-            for (int f = 0; f < F; ++f) term[4 + f] = gch[p][5 + f];
             float4 *row = reinterpret_cast<float4 *>(s_g + (p * 32 + lane) * WL::GROW);
+            row[0] = make_float4(gch[p][1].y, gch[p][0].x, gch[p][0].y, gch[p][1].x);
 #pragma unroll
-            for (int c = 0; c < WL::NWT / 4; ++c)
-                row[c] = make_float4(term[4 * c], term[4 * c + 1], term[4 * c + 2], term[4 * c + 3]);
+            for (int c = 0; c < F4; ++c)
+                row[1 + c] = make_float4(gch[p][2 + 2 * c].x, gch[p][2 + 2 * c].y, gch[p][3 + 2 * c].x, gch[p][3 + 2 * c].y);
         }
     }
 
-    // Map mode, after a stage of cnt splats: lane (column col, slot group jg) sums, for slots
-    // jg SPL + sj, w times the weighted terms [T0, T1) and (with MOM) dpow times (1, ly, ly^2) over
-    // the pixels of its column (eight distinct 16-byte rows per quarter-warp read), scales the
-    // column sums by the column's coordinate into the six moments, and the eight columns are
-    // added by a transpose reduction, lane col keeping block col of the chunk's sums.
+    // After a stage: lane (column col, slot group jg) sums, for its SPL slots, w times the weighted terms
+    // [T0, T1) and (with MOM) dpow times (1, dy, dy^2) down the pixels of its column, dy from the
+    // splat's own centre (so nothing cancels when the sums are formed), and scales the column sums by
+    // the column's dx into the moments.  Lanes of odd columns take the two halves of their slots in
+    // the opposite order, so that the first level of the transpose reduction over the eight columns
+    // sends one half and keeps the other without selects; the next two levels split the values.
     auto contract_chunk = [&](auto t0c, auto t1c, auto momc) {
         constexpr int T0 = decltype(t0c)::value, T1 = decltype(t1c)::value;
         constexpr bool MOM = decltype(momc)::value != 0;
-        constexpr int NT = T1 - T0, CV = NT + (MOM ? 6 : 0);
-        constexpr int CVP = (WL::SPL * CV + 7) / 8 * 8;
+        constexpr int SPL = WL::SPL, NT = T1 - T0, CV = NT + (MOM ? 6 : 0);
+        constexpr int HALF = SPL / 2 * CV, LEN = (HALF + 3) / 4 * 4;  // values kept after the first level
         const int col = lane & 7, jg = lane >> 3;
-        float acc[CVP];
+        const bool odd = col & 1;
+        float2 acc[SPL][NT / 2 > 0 ? NT / 2 : 1];
+        float s1[SPL], sy[SPL], syy[SPL], sd[SPL], dy[SPL], dx[SPL];
+        const float2 *wp[SPL];
 #pragma unroll
-        for (int c = 0; c < CVP; ++c) acc[c] = 0.f;
+        for (int sj = 0; sj < SPL; ++sj) {
+            const int j = jg * SPL + (odd ? (sj + SPL / 2) % SPL : sj);
+            wp[sj] = s_wp + j * WL::WROW + col;
 #pragma unroll
+            for (int c = 0; c < NT / 2; ++c) acc[sj][c] = make_float2(0.f, 0.f);
+            s1[sj] = sy[sj] = syy[sj] = sd[sj] = 0.f;
+            if constexpr (MOM) {
+                const float2 ctr = s_ctr[j];
+                dx[sj] = (float)col - 3.5f - ctr.x;
+                dy[sj] = 0.5f - 0.5f * WL::ROWS - ctr.y;
+            }
+        }
+#pragma unroll 4
         for (int ly = 0; ly < WL::ROWS; ++ly) {
-            const int q = ly * 8 + col;
-            const float lyc = (float)ly + 0.5f - 0.5f * WL::ROWS;
-            float w[WL::SPL];
+            float2 e[SPL];
 #pragma unroll
-            for (int sj = 0; sj < WL::SPL; ++sj) {
-                const int j = jg * WL::SPL + sj;
-                w[sj] = s_w[j * WL::WROW + q];
+            for (int sj = 0; sj < SPL; ++sj) {
+                e[sj] = wp[sj][ly * 8];
                 if constexpr (MOM) {
-                    const float dp = s_p[j * WL::WROW + q];
-                    float *a = acc + sj * CV + NT;
-                    a[0] += dp;
-                    a[1] = fmaf(lyc, dp, a[1]);
-                    a[2] = fmaf(lyc * lyc, dp, a[2]);
+                    const float d = dy[sj] + (float)ly, t = d * e[sj].y;
+                    s1[sj] += e[sj].y;
+                    sy[sj] += t;
+                    syy[sj] = fmaf(d, t, syy[sj]);
+                    if constexpr (!MAP) sd[sj] += e[sj].x;
                 }
             }
-            const float4 *g4 = reinterpret_cast<const float4 *>(s_g + q * WL::GROW + T0);
+            const float4 *g4 = reinterpret_cast<const float4 *>(s_g + (ly * 8 + col) * WL::GROW + T0);
 #pragma unroll
             for (int c = 0; c < NT / 4; ++c) {
                 const float4 gv = g4[c];
 #pragma unroll
-                for (int sj = 0; sj < WL::SPL; ++sj) {
-                    float *a = acc + sj * CV + 4 * c;
-                    a[0] = fmaf(w[sj], gv.x, a[0]);
-                    a[1] = fmaf(w[sj], gv.y, a[1]);
-                    a[2] = fmaf(w[sj], gv.z, a[2]);
-                    a[3] = fmaf(w[sj], gv.w, a[3]);
+                for (int sj = 0; sj < SPL; ++sj) {
+                    const float2 w = make_float2(e[sj].x, e[sj].x);
+                    acc[sj][2 * c] = fma2(w, make_float2(gv.x, gv.y), acc[sj][2 * c]);
+                    acc[sj][2 * c + 1] = fma2(w, make_float2(gv.z, gv.w), acc[sj][2 * c + 1]);
                 }
             }
         }
-        if constexpr (MOM) {
-            // column sums of dpow (1, ly, ly^2) -> moments (1, lx, ly, lx^2, lx ly, ly^2)
-            const float lxc = (float)col - 3.5f;
+        float v[LEN];
 #pragma unroll
-            for (int sj = 0; sj < WL::SPL; ++sj) {
-                float *a = acc + sj * CV + NT;
-                const float c0 = a[0], c1 = a[1], c2 = a[2];
-                a[1] = lxc * c0;
-                a[2] = c1;
-                a[3] = lxc * lxc * c0;
-                a[4] = lxc * c1;
-                a[5] = c2;
+        for (int i = 0; i < LEN; ++i) v[i] = 0.f;
+#pragma unroll
+        for (int sj = 0; sj < SPL; ++sj) {
+            float x[CV];
+#pragma unroll
+            for (int c = 0; c < NT / 2; ++c) {
+                x[2 * c] = acc[sj][c].x;
+                x[2 * c + 1] = acc[sj][c].y;
+            }
+            if constexpr (MOM) {
+                constexpr int M = MAP ? NT + 1 : 0;
+                if constexpr (MAP) x[NT] = s1[sj];
+                else x[5] = sd[sj];
+                const float sx = dx[sj] * s1[sj];
+                x[M] = sx;
+                x[M + 1] = sy[sj];
+                x[M + 2] = dx[sj] * sx;
+                x[M + 3] = dx[sj] * sy[sj];
+                x[M + 4] = syy[sj];
+            }
+            // slots of the second half go to the neighbouring column, whose second half arrives here
+#pragma unroll
+            for (int i = 0; i < CV; ++i) {
+                const int at = (sj % (SPL / 2)) * CV + i;
+                if (sj < SPL / 2) v[at] += x[i];
+                else v[at] += __shfl_xor_sync(0xffffffffu, x[i], 1);
             }
         }
-        // transpose reduction over the eight columns (lanes xor 4, 2, 1)
 #pragma unroll
-        for (int sft = 4, len = CVP; sft >= 1; sft >>= 1, len >>= 1) {
+        for (int sft = 2, len = LEN; sft <= 4; sft <<= 1, len >>= 1) {
             const bool up = col & sft;
 #pragma unroll
             for (int i = 0; i < len / 2; ++i) {
-                const float send = up ? acc[i] : acc[i + len / 2];
-                const float keep = up ? acc[i + len / 2] : acc[i];
-                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, sft);
+                const float send = up ? v[i] : v[i + len / 2];
+                const float keep = up ? v[i + len / 2] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, sft);
             }
         }
+        const int first = (col & 2 ? LEN / 2 : 0) + (col & 4 ? LEN / 4 : 0);
 #pragma unroll
-        for (int i = 0; i < CVP / 8; ++i) {
-            const int v = col * (CVP / 8) + i, sj = v / CV, t = v % CV;
-            if (v < WL::SPL * CV) s_t[(jg * WL::SPL + sj) * WL::NSV + (t < NT ? T0 + t : WL::NWT + t - NT)] = acc[i];
+        for (int i = 0; i < LEN / 4; ++i) {
+            const int q = first + i, sj = q / CV, t = q % CV;
+            if (q < HALF)
+                s_t[(jg * SPL + (odd ? SPL / 2 : 0) + sj) * WL::NSV + (t < NT ? T0 + t : WL::NWT + t - NT)] = v[i];
         }
     };
     // Then lanes (slot j, part) send slot j's sums to the splat's accumulators.
@@ -295,56 +328,48 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
         const int j = lane % STAGE, part = lane / STAGE;
         if (j < cnt) {
             const int64_t item = s_item[j];
-            const int64_t g = item - voff;
-            // slot j's sums: the terms (depth, r, g, b, F) then the moments (S1, Sx, Sy, Sxx, Sxy, Syy)
-            const float *tj = s_t + j * WL::NSV;
-            const float m1 = tj[WL::NWT], mx = tj[WL::NWT + 1], my = tj[WL::NWT + 2];
-            const float mxx = tj[WL::NWT + 3], mxy = tj[WL::NWT + 4], myy = tj[WL::NWT + 5];
+            // slot j's sums: the terms (depth, r, g, b, F) then the moments about the splat centre
+            const float *tj = s_t + j * WL::NSV, *mj = tj + WL::NWT + (MAP ? 1 : 0);
             if (part == 0) {
-                // centre and opacity from the moments expanded about the splat centre; depth
                 const SplatGeo sg = s_geo[j];
-                const float cx = __fadd_rn(__fsub_rn(sg.u, bcx), sg.ulo), cy = __fadd_rn(__fsub_rn(sg.v, bcy), sg.vlo);
-                const float Mx = fmaf(-cx, m1, mx), My = fmaf(-cy, m1, my);
-                const float du = (-1.f / kLog2e) * fmaf(2.f * sg.qa, Mx, sg.qb * My);
-                const float dv = (-1.f / kLog2e) * fmaf(2.f * sg.qc, My, sg.qb * Mx);
-                const float4 val = make_float4(du, dv, m1 / sg.o, tj[0]);
+                const float du = (-1.f / kLog2e) * fmaf(2.f * sg.qa, mj[0], sg.qb * mj[1]);
+                const float dv = (-1.f / kLog2e) * fmaf(2.f * sg.qc, mj[1], sg.qb * mj[0]);
+                const float4 val = MAP ? make_float4(du, dv, tj[WL::NWT] / sg.o, tj[0]) : make_float4(du, dv, 0.f, mj[5]);
                 if (val.x != 0.f || val.y != 0.f || val.z != 0.f || val.w != 0.f) atomicAdd(A.acc_uvod + item, val);
             } else if (part == 1) {
-                const SplatGeo sg = s_geo[j];
-                const float cx = __fadd_rn(__fsub_rn(sg.u, bcx), sg.ulo), cy = __fadd_rn(__fsub_rn(sg.v, bcy), sg.vlo);
-                // sum dpow dx^2 = Sxx - 2 cx Sx + cx^2 S1, and likewise
-                const float Mxx = fmaf(-cx, fmaf(-cx, m1, 2.f * mx), mxx);
-                const float Mxy = fmaf(cx * cy, m1, fmaf(-cx, my, fmaf(-cy, mx, mxy)));
-                const float Myy = fmaf(-cy, fmaf(-cy, m1, 2.f * my), myy);
-                const float4 val = make_float4(-0.5f * Mxx, -Mxy, -0.5f * Myy, 0.f);
+                const float4 val = make_float4(-0.5f * mj[2], -mj[3], -0.5f * mj[4], 0.f);
                 if (val.x != 0.f || val.y != 0.f || val.z != 0.f) atomicAdd(A.acc_conic + item, val);
             }
-            if (part == (WL::LPS > 2 ? 2 : 0)) {
-                const float4 val = make_float4(tj[1], tj[2], tj[3], 0.f);
-                if (val.x != 0.f || val.y != 0.f || val.z != 0.f) atomicAdd(A.acc_rgb + g, val);
-            }
-            // features [part D / LPS, (part + 1) D / LPS): the summed feature terms, or W^T times the
-            // summed logit terms
-            constexpr int DP = D / WL::LPS;
-            float *fo = A.d_feat + g * D + part * DP;
-#pragma unroll
-            for (int c4 = 0; c4 < DP / 4; ++c4) {
-                float o4[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int c = part * DP + 4 * c4 + i;
-                    if constexpr (KF > 0) {
-                        float sacc = 0.f;
-#pragma unroll
-                        for (int k = 0; k < KF; ++k) sacc = fmaf(s_basis[k * BROW + c], tj[4 + k], sacc);
-                        o4[i] = sacc;
-                    } else {
-                        o4[i] = tj[4 + c];
-                    }
+            if constexpr (MAP) {
+                const int64_t g = item - voff;
+                if (part == (WL::LPS > 2 ? 2 : 0)) {
+                    const float4 val = make_float4(tj[1], tj[2], tj[3], 0.f);
+                    if (val.x != 0.f || val.y != 0.f || val.z != 0.f) atomicAdd(A.acc_rgb + g, val);
                 }
-                const float4 val = make_float4(o4[0], o4[1], o4[2], o4[3]);
-                if (val.x != 0.f || val.y != 0.f || val.z != 0.f || val.w != 0.f)
-                    atomicAdd(reinterpret_cast<float4 *>(fo) + c4, val);
+                // features [part D / LPS, (part + 1) D / LPS): the summed feature terms, or W^T times the
+                // summed logit terms
+                constexpr int DP = D / WL::LPS;
+                float *fo = A.d_feat + g * D + part * DP;
+#pragma unroll
+                for (int c4 = 0; c4 < DP / 4; ++c4) {
+                    const int c = part * DP + 4 * c4;
+                    float4 val;
+                    if constexpr (KF > 0) {
+                        float2 lo = make_float2(0.f, 0.f), hi = lo;
+#pragma unroll
+                        for (int k = 0; k < KF; ++k) {
+                            const float4 b = *reinterpret_cast<const float4 *>(s_basis + k * BROW + c);
+                            const float2 z = make_float2(tj[4 + k], tj[4 + k]);
+                            lo = fma2(z, make_float2(b.x, b.y), lo);
+                            hi = fma2(z, make_float2(b.z, b.w), hi);
+                        }
+                        val = make_float4(lo.x, lo.y, hi.x, hi.y);
+                    } else {
+                        val = make_float4(tj[4 + c], tj[5 + c], tj[6 + c], tj[7 + c]);
+                    }
+                    if (val.x != 0.f || val.y != 0.f || val.z != 0.f || val.w != 0.f)
+                        atomicAdd(reinterpret_cast<float4 *>(fo) + c4, val);
+                }
             }
         }
         __syncwarp();
@@ -363,18 +388,17 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
             e[p] = eval_pair(s, pxc[p], pyc[p], prm.alpha_min, prm.alpha_max);
             contrib[p] = pos < last[p] && !e[p].skip;
         }
-        float val[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) val[i] = 0.f;
-        float x[NCH];
+        float2 x[NC2];
         {
             const float4 c = s_rgbd[k];
-            x[0] = c.x; x[1] = c.y; x[2] = c.z; x[3] = c.w; x[4] = 1.f;
+            x[0] = make_float2(c.x, c.y);
+            x[1] = make_float2(c.z, c.w);
             const float4 *sf = reinterpret_cast<const float4 *>(sfeat + k * fstride);
 #pragma unroll
             for (int q = 0; q < F4; ++q) {
                 const float4 f = sf[q];
-                x[5 + 4 * q] = f.x; x[6 + 4 * q] = f.y; x[7 + 4 * q] = f.z; x[8 + 4 * q] = f.w;
+                x[2 + 2 * q] = make_float2(f.x, f.y);
+                x[3 + 2 * q] = make_float2(f.z, f.w);
             }
         }
         // Branch-free over the lanes: a pixel that did not blend the splat runs the same
@@ -383,43 +407,21 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
         for (int p = 0; p < NP; ++p) {
             const float a = contrib[p] ? e[p].alpha : 0.f;
             const float Tb = __fdividef(T[p], 1.f - a);
-            // g.x as three interleaved partial sums (shorter dependent chain)
-            float gx3[3] = {0.f, 0.f, 0.f};
+            // g.x as four interleaved partial sums, two packed (a short dependent chain)
+            float2 ga = make_float2(gsil[p], 0.f), gb = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) gx3[ch % 3] = fmaf(gch[p][ch], x[ch], gx3[ch % 3]);
-            const float gx = gx3[0] + gx3[1] + gx3[2];
+            for (int c = 0; c < NC2; c += 2) {
+                ga = fma2(gch[p][c], x[c], ga);
+                gb = fma2(gch[p][c + 1], x[c + 1], gb);
+            }
+            const float gx = (ga.x + ga.y) + (gb.x + gb.y);
             const float da = Tb * (gx - gS[p]);
             gS[p] = fmaf(a, gx - gS[p], gS[p]);
             T[p] = contrib[p] ? Tb : T[p];
             const bool free_alpha = contrib[p] && e[p].oG < prm.alpha_max;
-            const float dpow = free_alpha ? e[p].oG * da : 0.f;
-            if constexpr (MAP) {
-                s_w[k * WL::WROW + p * 32 + lane] = a * Tb;
-                s_p[k * WL::WROW + p * 32 + lane] = dpow;
-            } else {
-                // moments of dpow over the pixels; the splat's constants scale them once, after
-                // the warp reduction (geo_grads); the depth term as the sixth value
-                const float dx = e[p].dx, dy = e[p].dy;
-                const float ax = dx * dpow, ay = dy * dpow;
-                val[0] += ax;
-                val[1] += ay;
-                val[2] = fmaf(ax, dx, val[2]);
-                val[3] = fmaf(ax, dy, val[3]);
-                val[4] = fmaf(ay, dy, val[4]);
-                val[5] = fmaf(a * Tb, gch[p][3], val[5]);
-            }
-        }
-        if constexpr (!MAP) {
-            // lane i ends with the warp's value (i mod 8): centre (0, 1), conic (2-4), depth (5); lanes
-            // 0-5 add them in one warp-wide reduction instruction
-            const uint32_t item = s_item[k];
-            const float r = geo_grads(warp_transpose_reduce<8>(val, lane), lane & 7, s);
-            if (lane < 6 && r != 0.f) {
-                float *dst = lane == 5 ? reinterpret_cast<float *>(A.acc_uvod + item) + 3
-                             : lane < 2 ? reinterpret_cast<float *>(A.acc_uvod + item) + lane
-                                        : reinterpret_cast<float *>(A.acc_conic + item) + (lane - 2);
-                atomicAdd(dst, r);
-            }
+            const float w = a * Tb;
+            s_wp[k * WL::WROW + p * 32 + lane] =
+                make_float2(MAP ? w : w * gch[p][1].y, free_alpha ? e[p].oG * da : 0.f);
         }
     };
 
@@ -469,7 +471,9 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
                 const int64_t g = (int64_t)item - voff;
                 if (part == 0) {
                     const float4 a = r_a[b][si];
-                    s_geo[si] = make_geo(a, r_lo[b][si], r_c[b][si]);
+                    const float2 l = r_lo[b][si];
+                    s_geo[si] = make_geo(a, l, r_c[b][si]);
+                    s_ctr[si] = make_float2(__fadd_rn(__fsub_rn(a.x, bcx), l.x), __fadd_rn(__fsub_rn(a.y, bcy), l.y));
                     s_rgbd[si] = RGB32 ? make_float4(r_rgb[b][si][0], r_rgb[b][si][1], r_rgb[b][si][2], a.z)
                                        : load_rgbd(rgb, g, a.z);
                     s_item[si] = item;
@@ -481,17 +485,15 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
 #pragma unroll
                     for (int kk = 0; kk < KF / PARTS; ++kk) {
                         const int k = part * (KF / PARTS) + kk;
-                        float z = 0.f;
+                        float2 za = make_float2(0.f, 0.f), zb = za;
 #pragma unroll
                         for (int q = 0; q < D / 4; ++q) {
                             const float4 f4 = load_feat4(fr, 4 * q);
                             const float4 w4 = reinterpret_cast<const float4 *>(s_basis + k * BROW)[q];
-                            z = fmaf(w4.x, f4.x, z);
-                            z = fmaf(w4.y, f4.y, z);
-                            z = fmaf(w4.z, f4.z, z);
-                            z = fmaf(w4.w, f4.w, z);
+                            za = fma2(make_float2(w4.x, w4.y), make_float2(f4.x, f4.y), za);
+                            zb = fma2(make_float2(w4.z, w4.w), make_float2(f4.z, f4.w), zb);
                         }
-                        s_feat[si * F + k] = z;
+                        s_feat[si * F + k] = (za.x + za.y) + (zb.x + zb.y);
                     }
                 } else if (!RGB32 || sizeof(FT) != 4) {
                     // half storage: the features widened to f32
@@ -503,8 +505,11 @@ __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
             // f32 features are read where they landed; the others from the widened copy
             constexpr bool IN_PLACE = KF == 0 && sizeof(FT) == 4;
             const float *sfeat = IN_PLACE ? reinterpret_cast<const float *>(r_f[b]) : s_feat;
+            // two splats at a time overlap their loads and exponentials, where the registers allow
+            constexpr int kTogether = KF > 0 ? 2 : 1;
+#pragma unroll kTogether
             for (int k = 0; k < c_cnt; ++k) process(k, sfeat, IN_PLACE ? FBP / 4 : F);
-            if constexpr (MAP) contract(c_cnt);
+            contract(c_cnt);
             __syncwarp();
         }
     };

@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -22,67 +23,68 @@ namespace gs {
 namespace {
 
 constexpr int kMaxK = 32;
-
-// Block-wide (256 threads) exclusive scan of one u32 per thread.
-__device__ __forceinline__ uint32_t scan256(uint32_t x, uint32_t *total, uint32_t *s_warp) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t inc = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    if (lane == 31) s_warp[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        const uint32_t t = lane < 8 ? s_warp[lane] : 0;
-        uint32_t ti = t;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, ti, o);
-            if (lane >= o) ti += y;
-        }
-        if (lane < 8) s_warp[lane] = ti - t;
-        if (lane == 7) s_warp[8] = ti;
-    }
-    __syncthreads();
-    const uint32_t r = s_warp[w] + inc - x;
-    *total = s_warp[8];
-    __syncthreads();
-    return r;
-}
+constexpr int kMedianBlocks = 1024;  // of a pass of the median's histograms, over all views
 
 // Lower median (element floor((n-1)/2) in sorted order) of view v, as the f32
 // bit pattern selected digit by digit from the per-pass histograms
-// hist[p][v][256] (p < passes); the whole 256-thread block cooperates.
-__device__ uint32_t block_select(const uint32_t *hist, int n_views, int v, int passes) {
-    __shared__ uint32_t s_warp[9];
-    __shared__ uint32_t s_k, s_prefix, s_sel, s_below;
-    const int d = threadIdx.x;
-    uint32_t n;
-    scan256(hist[(size_t)v * 256 + d], &n, s_warp);
-    if (d == 0) {
-        s_k = n > 0 ? (n - 1) / 2 : 0;
-        s_prefix = 0;
+// hist[p][v][256] (p < passes), by one warp: lane l holds digits [8 l, 8 l + 8) of every pass, loaded
+// together (the passes' counts do not depend on one another once written), and each pass takes
+// one scan over the lanes.  Valid in every lane.
+__device__ __forceinline__ uint32_t warp_select(const uint32_t *hist, int n_views, int v, int passes) {
+    const int lane = threadIdx.x & 31;
+    uint32_t h[4][8];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(hist + ((size_t)p * n_views + v) * 256 + 8 * lane);
+        const uint4 z = make_uint4(0u, 0u, 0u, 0u), a = p < passes ? src[0] : z, b = p < passes ? src[1] : z;
+        h[p][0] = a.x; h[p][1] = a.y; h[p][2] = a.z; h[p][3] = a.w;
+        h[p][4] = b.x; h[p][5] = b.y; h[p][6] = b.z; h[p][7] = b.w;
+    }
+    uint32_t k = 0u, prefix = 0u;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        uint32_t sum = 0u;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sum += h[p][i];
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (p == 0) {
+            const uint32_t n = __shfl_sync(0xffffffffu, inc, 31);
+            if (n == 0u) return 0u;  // no pixel with depth
+            k = (n - 1u) / 2u;
+        }
+        if (p >= passes) break;
+        // the lane whose digits hold element k, the digit, and the elements below it
+        uint32_t below = inc - sum, digit = 0u, rest = 0u;
+        const uint32_t owner = __ballot_sync(0xffffffffu, k >= below && k < inc);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (k >= below && k < below + h[p][i]) {
+                digit = 8u * lane + i;
+                rest = below;
+            }
+            below += h[p][i];
+        }
+        const int src = __ffs(owner) - 1;
+        digit = __shfl_sync(0xffffffffu, digit, src);
+        k -= __shfl_sync(0xffffffffu, rest, src);
+        prefix |= digit << (24 - 8 * p);
+    }
+    return prefix;
+}
+
+// The same for a block (every thread of it takes part).
+__device__ __forceinline__ uint32_t block_select(const uint32_t *hist, int n_views, int v, int passes) {
+    __shared__ uint32_t s_prefix;
+    if (threadIdx.x < 32) {
+        const uint32_t x = warp_select(hist, n_views, v, passes);
+        if (threadIdx.x == 0) s_prefix = x;
     }
     __syncthreads();
-    if (n == 0) return 0;
-    for (int p = 0; p < passes; ++p) {
-        const uint32_t h = hist[((size_t)p * n_views + v) * 256 + d];
-        uint32_t tot;
-        const uint32_t ex = scan256(h, &tot, s_warp);
-        const uint32_t k = s_k;
-        if (k >= ex && k < ex + h) {
-            s_sel = d;
-            s_below = ex;
-        }
-        __syncthreads();
-        if (d == 0) {
-            s_prefix |= s_sel << (24 - 8 * p);
-            s_k = k - s_below;
-        }
-        __syncthreads();
-    }
     return s_prefix;
 }
 
@@ -90,25 +92,26 @@ __device__ __forceinline__ float depth_error(float d, float dgt) { return fabsf(
 
 __global__ void __launch_bounds__(256) median_hist_kernel(ViewTable vt, int pass, const float *depth,
                                                           const float *tdepth, uint32_t *hist) {
+    pdl_wait();     // the previous kernel's results
+    pdl_trigger();  // the next kernel may be scheduled now
     __shared__ uint32_t s_hist[256];
-    __shared__ uint32_t s_prefix;
     const int v = blockIdx.y;
     const int64_t Pv = (int64_t)vt.W[v] * vt.H[v];
     s_hist[threadIdx.x] = 0;
-    const uint32_t pre = pass > 0 ? block_select(hist, vt.n_views, v, pass) : 0u;
-    if (threadIdx.x == 0) s_prefix = pre;
+    const uint32_t prefix = pass > 0 ? block_select(hist, vt.n_views, v, pass) : 0u;
     __syncthreads();
     const int lane = threadIdx.x & 31;
+#pragma unroll 4
     for (int64_t base = (int64_t)blockIdx.x * 256; base < Pv; base += (int64_t)gridDim.x * 256) {
         const int64_t i = base + threadIdx.x;
         bool valid = false;
         uint32_t bits = 0;
         if (i < Pv) {
             const int64_t pix = vt.pix_off[v] + i;
-            const float dgt = tdepth[pix];
+            const float dgt = tdepth[pix], d = depth[pix];
             if (dgt > 0.f) {
-                bits = __float_as_uint(depth_error(depth[pix], dgt));
-                valid = pass == 0 || (bits >> (32 - 8 * pass)) == (s_prefix >> (32 - 8 * pass));
+                bits = __float_as_uint(depth_error(d, dgt));
+                valid = pass == 0 || (bits >> (32 - 8 * pass)) == (prefix >> (32 - 8 * pass));
             }
         }
         const uint32_t dg = valid ? (bits >> (24 - 8 * pass)) & 255u : 256u + lane;
@@ -118,6 +121,17 @@ __global__ void __launch_bounds__(256) median_hist_kernel(ViewTable vt, int pass
     __syncthreads();
     const uint32_t c = s_hist[threadIdx.x];
     if (c) atomicAdd(&hist[((size_t)pass * vt.n_views + v) * 256 + threadIdx.x], c);
+}
+
+// The four passes of the median's histograms (hist zeroed here), each launched while its predecessor
+// drains.
+gs_status launch_median(const ViewTable &vt, const float *depth, const float *tdepth, uint32_t *hist, int blocks_x,
+                        cudaStream_t st) {
+    gs_status s = cuda_status(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * 4 * 256 * vt.n_views, st));
+    const dim3 grid(blocks_x, vt.n_views);
+    for (int pass = 0; pass < 4 && !s; ++pass)
+        s = launch_pdl(median_hist_kernel, grid, 256, 0, st, vt, pass, depth, tdepth, hist);
+    return s;
 }
 
 struct LossP {
@@ -145,6 +159,39 @@ __device__ __forceinline__ float warp_transpose_reduce(float (&v)[N], int lane) 
     return r;
 }
 
+// Sums of N per-thread f32 values over the block in f64 (thread i's value x[n], rounding error lo[n]
+// subtracted where LO), in a fixed order; out[n] valid in every thread.  The values go through
+// shared memory and one warp adds each sum: NT / 32 additions and five shuffle steps for 32 threads
+// instead of five steps for all of them, since the GPU adds two f64 a cycle and SM (the loss kernel's
+// three sums with a division in every thread kept its blocks for 7 of 45 us).
+template <int NT, bool LO, int N>
+__device__ __forceinline__ void block_sums_f64(const float (&x)[N], const float *lo, double (&out)[N]) {
+    __shared__ float s_x[LO ? 2 : 1][N][NT];
+    __shared__ double s_sum[N];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    __syncthreads();
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        s_x[0][n][tid] = x[n];
+        if constexpr (LO) s_x[LO][n][tid] = lo[n];
+    }
+    __syncthreads();
+    for (int n = w; n < N; n += NT / 32) {
+        double t = 0.0;
+#pragma unroll
+        for (int i = 0; i < NT / 32; ++i) {
+            t += (double)s_x[0][n][i * 32 + lane];
+            if constexpr (LO) t -= (double)s_x[LO][n][i * 32 + lane];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) s_sum[n] = t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int n = 0; n < N; ++n) out[n] = s_sum[n];
+}
+
 // Sum over the block (any multiple of 32 threads, up to 1024) in f64; valid in thread 0.
 __device__ __forceinline__ double block_sum_f64(double x, double *s_red) {
 #pragma unroll
@@ -159,28 +206,47 @@ __device__ __forceinline__ double block_sum_f64(double x, double *s_red) {
     return t;
 }
 
+// Blocks [off[v], off[v + 1]) of the loss kernel's grid work on view v.
+struct LossGrid {
+    int off[kMaxViews + 1];
+};
+
 // Per-pixel losses and image gradients; per-block partials of the decoder
 // gradient (f32 [nblk][K*D + K]) and of the three loss sums (f64 [nblk][3]).
 //
-// KC is a compile-time bound on the class count (K <= KC).  The decoder
-// gradient dW[k][d] = sum_px dz_k f_d, db[k] = sum_px dz_k is a contraction over
-// pixels: each warp stages dz and f of its 32 pixels in shared memory, and every
-// lane keeps EPL consecutive entries of one row of dW (lanes < KC also one
-// entry of db) in registers for the whole grid-stride loop; they reach the
-// block's shared sums once, at the end.
+// KC is a compile-time bound on the class count (K <= KC, a multiple of 8).  What bounds the kernel
+// is the shared-memory pipe (a 16-byte read costs a warp four cycles even as a broadcast) and its
+// FMAs, so that each word read serves as many of them as registers allow:
+//  - a thread takes NPX pixels at a time, so each row of W read for z = W f and W^T dz serves
+//    NPX of them, in packed multiply-adds along d;
+//  - the decoder gradient dW[k][d] = sum_px dz_k f_d, db[k] = sum_px dz_k is a contraction over pixels:
+//    each warp stages dz and f of 32 pixels in shared memory, and every lane keeps an 8 x 4 tile
+//    of dW in registers for the whole grid-stride loop (TILES lanes cover K x D, GROUPS such
+//    sets of lanes each take their share of the 32 pixels): 12 words read for 32 multiply-adds.
+//    The sums reach the block's shared ones once, at the end.
+// Loss step (this kernel and the finish), before and now: 0.054 -> 0.047 ms (D = 16, K = 8, 1200x680),
+// 0.433 -> 0.25 (D = 32, K = 8, eight keyframes of two sizes), 0.167 -> 0.096 (D = 16, K = 20, 1200x680, with
+// the features' gradient).  Two pixels a thread where 128 registers hold them without spilling (K = 20:
+// 0.101 with two, 0.096 with one).
 template <int D, int KC>
 struct LossShape {
-    static constexpr int NT = (KC <= 8 && D <= 16) ? 256 : 128;  // keeps the static shared memory < 48 KB
+    static constexpr int NT = 128;                        // keeps the static shared memory < 48 KB
+    static constexpr int NPX = KC + D <= 32 ? 2 : 1;      // pixels a thread has in flight
+    // resident blocks the register allocation must allow (128 registers, 168 for the widest)
+    static constexpr int BLOCKS = KC + D > 40 || (NPX == 2 && KC >= 16 && KC + D >= 28) ? 3 : 4;
     static constexpr int WARPS = NT / 32;
     static constexpr int DD = D > 0 ? D : 1;
-    static constexpr int EPL = D > 0 ? KC * D / 32 : 1;          // dW entries per lane
-    static constexpr int FROW = D > 0 ? D + 4 : 4;              // staged feature row (16-byte aligned, padded)
-    static_assert(D == 0 || ((KC * D) % 32 == 0 && D % EPL == 0), "lane blocks of dW");
+    static constexpr int D4 = D / 4 > 0 ? D / 4 : 1;
+    static constexpr int FROW = D > 0 ? D + 4 : 4;        // staged rows, padded: eight lanes' 16-byte
+    static constexpr int ZROW = KC + 4;                   // words of neighbouring rows fall in different banks
+    static constexpr int TILES = KC / 8 * D4;
+    static constexpr int GROUPS = TILES <= 4 ? 8 : TILES <= 8 ? 4 : TILES <= 16 ? 2 : 1;
+    static_assert(KC % 8 == 0 && D % 4 == 0 && TILES * GROUPS <= 32, "8 x 4 tiles of dW");
 };
 
 template <int D, int KC>
-__global__ void __launch_bounds__(LossShape<D, KC>::NT) loss_kernel(
-    ViewTable vt, LossP lp, const float *__restrict__ rgb, const float *__restrict__ depth,
+__global__ void __launch_bounds__(LossShape<D, KC>::NT, LossShape<D, KC>::BLOCKS) loss_kernel(
+    ViewTable vt, LossGrid lg, LossP lp, const float *__restrict__ rgb, const float *__restrict__ depth,
     const float *__restrict__ sil, const float *__restrict__ feat, const float *__restrict__ trgb,
     const float *__restrict__ tdepth, const uint8_t *__restrict__ label, const float *__restrict__ Wd,
     const float *__restrict__ bd, int64_t P, const uint32_t *__restrict__ med_hist, float *__restrict__ g_rgb,
@@ -190,207 +256,275 @@ __global__ void __launch_bounds__(LossShape<D, KC>::NT) loss_kernel(
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
     using SH = LossShape<D, KC>;
-    constexpr int NT = SH::NT, DD = SH::DD, EPL = SH::EPL;
+    constexpr int NT = SH::NT, NPX = SH::NPX, DD = SH::DD, TILES = SH::TILES, GROUPS = SH::GROUPS;
     __shared__ __align__(16) float s_W[KC * DD];
     __shared__ float s_b[KC];
     __shared__ float s_dW[KC * DD + KC];
-    __shared__ float s_dz[SH::WARPS][32][KC + 1];
+    __shared__ __align__(16) float s_dz[SH::WARPS][32][SH::ZROW];
     __shared__ __align__(16) float s_f[SH::WARPS][32][SH::FROW];
-    __shared__ double s_red[8];
     __shared__ float s_med;
-    const int v = blockIdx.y;
-    const int blk = v * gridDim.x + blockIdx.x;
+    const int blk = blockIdx.x;
+    int v = 0;
+    while (v + 1 < vt.n_views && blk >= lg.off[v + 1]) ++v;
+    const int bx = blk - lg.off[v], nbx = lg.off[v + 1] - lg.off[v];
     const int64_t Pv = (int64_t)vt.W[v] * vt.H[v];
     const int K = lp.K, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nval = K * D + K;
-    for (int i = tid; i < K * D; i += NT) s_W[i] = Wd[i];
+    for (int i = tid; i < KC * D; i += NT) s_W[i] = i < K * D ? Wd[i] : 0.f;
     for (int i = tid; i < K; i += NT) s_b[i] = bd[i];
     for (int i = tid; i < nval; i += NT) s_dW[i] = 0.f;
-    float med = 0.f;
-    if (lp.mask_mode == 1) med = __uint_as_float(block_select(med_hist, vt.n_views, v, 4));
-    if (tid == 0) {
-        s_med = med;
-        if (median_out && blockIdx.x == 0) median_out[v] = med;
+    if (wid == 0) {
+        const float med = lp.mask_mode == 1 ? __uint_as_float(warp_select(med_hist, vt.n_views, v, 4)) : 0.f;
+        if (lane == 0) {
+            s_med = med;
+            if (median_out && bx == 0) median_out[v] = med;
+        }
     }
     __syncthreads();
+    // the view's planes: uniform base addresses, so that a pixel's 32-bit index addresses every plane
+    const int64_t o = vt.pix_off[v];
+    rgb += o; depth += o; sil += o; trgb += o; tdepth += o; label += o; g_rgb += o; g_depth += o; g_sil += o;
+    if (D > 0) feat += o;
+    if (g_feat) g_feat += o;
+    if (g_coef) g_coef += o;
+    if (mask_out) mask_out += o;
+    const uint32_t n_px = (uint32_t)Pv;
     const float invP = 1.f / (float)Pv;
     float lc = 0.f, ld = 0.f, ls = 0.f;  // per-thread partial sums (a thread sees few pixels)
-    // this lane's decoder-gradient entries: dW[kr][d0, d0 + EPL) and db[lane]
-    const int kr = D > 0 ? (lane * EPL) / D : 0, d0 = D > 0 ? (lane * EPL) % D : 0;
-    float accW[EPL], accb = 0.f;
+    // this lane's tile of the decoder gradient: classes [k0, k0 + 8), features [d0, d0 + 4), pixel group grp
+    const int tile = lane % TILES, grp = lane / TILES;
+    const int k0 = tile / SH::D4 * 8, d0 = tile % SH::D4 * 4;
+    float2 accW[8][2], accb[4];
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) accW[e] = 0.f;
+    for (int k = 0; k < 8; ++k) accW[k][0] = accW[k][1] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) accb[k] = make_float2(0.f, 0.f);
 
-    // two pixels of the grid-stride loop in flight: the next one's loads issue beside this one's work
-#pragma unroll 2
-    for (int64_t base = (int64_t)blockIdx.x * NT; base < Pv; base += (int64_t)gridDim.x * NT) {
-        const int64_t i = base + tid;
-        float f[DD], dz[KC];
+    for (uint32_t base = (uint32_t)bx * (NT * NPX); base < n_px; base += (uint32_t)nbx * (NT * NPX)) {
+        float f[NPX][DD], dz[NPX][KC];
+        int lab[NPX];
+        float m[NPX];
+        // loads first: colours, depths, labels and features of the thread's pixels
 #pragma unroll
-        for (int k = 0; k < KC; ++k) dz[k] = 0.f;
+        for (int p = 0; p < NPX; ++p) {
+            const uint32_t i = base + p * NT + tid;
+            lab[p] = 255;
+            m[p] = 1.f;
 #pragma unroll
-        for (int d = 0; d < DD; ++d) f[d] = 0.f;
-        if (i < Pv) {
-            const int64_t pix = vt.pix_off[v] + i;
-            const float dgt = tdepth[pix], dd = depth[pix];
-            float m = 1.f;
-            if (lp.mask_mode == 1)
-                m = (sil[pix] > lp.tau_obs && dgt > 0.f && depth_error(dd, dgt) < 10.f * s_med) ? 1.f : 0.f;
-            if (mask_out) mask_out[pix] = m;
+            for (int d = 0; d < DD; ++d) f[p][d] = 0.f;
+            if (i < n_px) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const float r = rgb[c * P + pix] - trgb[c * P + pix];
-                lc += m * fabsf(r);
-                g_rgb[c * P + pix] = m * lp.color * (r > 0.f ? 1.f : (r < 0.f ? -1.f : 0.f)) * invP;
-            }
-            float gd = 0.f;
-            if (dgt > 0.f) {
-                const float r = dd - dgt;
-                ld += m * fabsf(r);
-                gd = m * lp.depth * (r > 0.f ? 1.f : (r < 0.f ? -1.f : 0.f)) * invP;
-            }
-            g_depth[pix] = gd;
-            g_sil[pix] = 0.f;
+                for (int d = 0; d < D; ++d) f[p][d] = (feat + d * P)[i];
+                lab[p] = label[i];
+                const float dgt = tdepth[i], dd = depth[i];
+                if (lp.mask_mode == 1)
+                    m[p] = (sil[i] > lp.tau_obs && dgt > 0.f && depth_error(dd, dgt) < 10.f * s_med) ? 1.f : 0.f;
+                if (mask_out) mask_out[i] = m[p];
 #pragma unroll
-            for (int d = 0; d < D; ++d) f[d] = feat[d * P + pix];
-            const int lab = label[pix];
-            if (lab != 255 && lab < K) {
-                // z = W f + b, each row read as float4 and summed in four partial sums
-                float z[KC];
-                float zmax = -INFINITY;
-#pragma unroll
-                for (int k = 0; k < KC; ++k) {
-                    z[k] = 0.f;
-                    if (k < K) {
-                        float a[4] = {0.f, 0.f, 0.f, 0.f};
-                        if constexpr (D % 4 == 0) {
-                            const float4 *wr = reinterpret_cast<const float4 *>(s_W + k * D);
-#pragma unroll
-                            for (int q = 0; q < D / 4; ++q) {
-                                const float4 w4 = wr[q];
-                                a[0] = fmaf(w4.x, f[4 * q], a[0]);
-                                a[1] = fmaf(w4.y, f[4 * q + 1], a[1]);
-                                a[2] = fmaf(w4.z, f[4 * q + 2], a[2]);
-                                a[3] = fmaf(w4.w, f[4 * q + 3], a[3]);
-                            }
-                        } else {
-#pragma unroll
-                            for (int d = 0; d < D; ++d) a[d & 3] = fmaf(s_W[k * D + d], f[d], a[d & 3]);
-                        }
-                        const float s = s_b[k] + ((a[0] + a[1]) + (a[2] + a[3]));
-                        z[k] = s;
-                        zmax = fmaxf(zmax, s);
-                    }
+                for (int c = 0; c < 3; ++c) {
+                    const float r = (rgb + c * P)[i] - (trgb + c * P)[i];
+                    lc += m[p] * fabsf(r);
+                    (g_rgb + c * P)[i] = m[p] * lp.color * (r > 0.f ? 1.f : (r < 0.f ? -1.f : 0.f)) * invP;
                 }
-                // softmax from one exponential per class: p_k = e_k / sum_j e_j, e_k = exp(z_k - zmax)
-                float e[KC], se = 0.f, zl = 0.f;
-#pragma unroll
-                for (int k = 0; k < KC; ++k) {
-                    e[k] = 0.f;
-                    if (k < K) {
-                        e[k] = expf(z[k] - zmax);
-                        se += e[k];
-                        if (k == lab) zl = z[k];
-                    }
+                float gd = 0.f;
+                if (dgt > 0.f) {
+                    const float r = dd - dgt;
+                    ld += m[p] * fabsf(r);
+                    gd = m[p] * lp.depth * (r > 0.f ? 1.f : (r < 0.f ? -1.f : 0.f)) * invP;
                 }
-                const float lse = zmax + logf(se);
-                ls += m * (lse - zl);
-                const float scale = m * lp.sem * invP;
-                const float inv_se = 1.f / se;
-#pragma unroll
-                for (int k = 0; k < KC; ++k)
-                    if (k < K) dz[k] = scale * (e[k] * inv_se - (k == lab ? 1.f : 0.f));
-            }
-            if (g_coef) {
-                // the factored feature gradient: dL/dz itself (g_feat = W^T dz is left to the backward)
-#pragma unroll
-                for (int k = 0; k < KC; ++k)
-                    if (k < K) g_coef[k * P + pix] = dz[k];
-            } else {
-                float gf[DD];
-#pragma unroll
-                for (int d = 0; d < DD; ++d) gf[d] = 0.f;
-#pragma unroll
-                for (int k = 0; k < KC; ++k) {
-                    if (k < K) {
-                        if constexpr (D % 4 == 0) {
-                            const float4 *wr = reinterpret_cast<const float4 *>(s_W + k * D);
-#pragma unroll
-                            for (int q = 0; q < D / 4; ++q) {
-                                const float4 w4 = wr[q];
-                                gf[4 * q] = fmaf(w4.x, dz[k], gf[4 * q]);
-                                gf[4 * q + 1] = fmaf(w4.y, dz[k], gf[4 * q + 1]);
-                                gf[4 * q + 2] = fmaf(w4.z, dz[k], gf[4 * q + 2]);
-                                gf[4 * q + 3] = fmaf(w4.w, dz[k], gf[4 * q + 3]);
-                            }
-                        } else {
-#pragma unroll
-                            for (int d = 0; d < D; ++d) gf[d] = fmaf(s_W[k * D + d], dz[k], gf[d]);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int d = 0; d < D; ++d) g_feat[d * P + pix] = gf[d];
+                g_depth[i] = gd;
+                g_sil[i] = 0.f;
             }
         }
-        if (K > 0) {
-            // stage the warp's dz and f, then accumulate this lane's dW / db entries over its 32 pixels
+        if (K == 0) {
+            if (!g_coef) {
 #pragma unroll
-            for (int k = 0; k < KC; ++k) s_dz[wid][lane][k] = dz[k];
+                for (int p = 0; p < NPX; ++p) {
+                    const uint32_t i = base + p * NT + tid;
+#pragma unroll
+                    for (int d = 0; d < D; ++d)
+                        if (i < n_px) (g_feat + d * P)[i] = 0.f;
+                }
+            }
+            continue;
+        }
+        // z = W f + b, each row summed in four partial sums (two packed)
+#pragma unroll
+        for (int k = 0; k < KC; ++k) {
+            if (k < K) {
+                float2 a[NPX][2];
+#pragma unroll
+                for (int p = 0; p < NPX; ++p) a[p][0] = a[p][1] = make_float2(0.f, 0.f);
+                if constexpr (D > 0) {
+                    const float4 *wr = reinterpret_cast<const float4 *>(s_W + k * D);
+#pragma unroll
+                    for (int q = 0; q < D / 4; ++q) {
+                        const float4 w4 = wr[q];
+#pragma unroll
+                        for (int p = 0; p < NPX; ++p) {
+                            a[p][0] = fma2(make_float2(w4.x, w4.y), make_float2(f[p][4 * q], f[p][4 * q + 1]), a[p][0]);
+                            a[p][1] = fma2(make_float2(w4.z, w4.w), make_float2(f[p][4 * q + 2], f[p][4 * q + 3]), a[p][1]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int p = 0; p < NPX; ++p) dz[p][k] = s_b[k] + ((a[p][0].x + a[p][0].y) + (a[p][1].x + a[p][1].y));
+            } else {
+#pragma unroll
+                for (int p = 0; p < NPX; ++p) dz[p][k] = 0.f;
+            }
+        }
+        // softmax from one exponential per class: p_k = e_k / sum_j e_j, e_k = exp(z_k - zmax)
+#pragma unroll
+        for (int p = 0; p < NPX; ++p) {
+            const bool on = lab[p] != 255 && lab[p] < K;
+            float zmax = -INFINITY, se = 0.f, zl = 0.f;
+#pragma unroll
+            for (int k = 0; k < KC; ++k)
+                if (k < K) {
+                    zmax = fmaxf(zmax, dz[p][k]);
+                    if (k == lab[p]) zl = dz[p][k];
+                }
+#pragma unroll
+            for (int k = 0; k < KC; ++k)
+                if (k < K) {
+                    dz[p][k] = expf(dz[p][k] - zmax);
+                    se += dz[p][k];
+                }
+            if (on) ls += m[p] * (zmax + logf(se) - zl);
+            const float scale = m[p] * lp.sem * invP;
+            const float inv_se = 1.f / se;
+#pragma unroll
+            for (int k = 0; k < KC; ++k)
+                if (k < K) dz[p][k] = on ? scale * (dz[p][k] * inv_se - (k == lab[p] ? 1.f : 0.f)) : 0.f;
+        }
+        // the decoder gradient: the warp's dz and f of 32 pixels staged, each lane's tile summed over its
+        // group's share of them
+#pragma unroll
+        for (int p = 0; p < NPX; ++p) {
+            float4 *zr = reinterpret_cast<float4 *>(&s_dz[wid][lane][0]);
+#pragma unroll
+            for (int q = 0; q < KC / 4; ++q)
+                zr[q] = make_float4(dz[p][4 * q], dz[p][4 * q + 1], dz[p][4 * q + 2], dz[p][4 * q + 3]);
             if constexpr (D > 0) {
                 float4 *fr = reinterpret_cast<float4 *>(&s_f[wid][lane][0]);
 #pragma unroll
-                for (int q = 0; q < D / 4; ++q) fr[q] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+                for (int q = 0; q < D / 4; ++q)
+                    fr[q] = make_float4(f[p][4 * q], f[p][4 * q + 1], f[p][4 * q + 2], f[p][4 * q + 3]);
             }
             __syncwarp();
-#pragma unroll 4
-            for (int px = 0; px < 32; ++px) {
-                if constexpr (D > 0) {
-                    const float zk = s_dz[wid][px][kr];
-                    if constexpr (EPL % 4 == 0) {
-                        const float4 *fr = reinterpret_cast<const float4 *>(&s_f[wid][px][d0]);
+            if (grp < GROUPS) {
+#pragma unroll 2
+                for (int it = 0; it < 32 / GROUPS; ++it) {
+                    const int px = grp * (32 / GROUPS) + it;
+                    const float4 za = *reinterpret_cast<const float4 *>(&s_dz[wid][px][k0]);
+                    const float4 zb = *reinterpret_cast<const float4 *>(&s_dz[wid][px][k0 + 4]);
+                    if constexpr (D > 0) {
+                        const float4 fv = *reinterpret_cast<const float4 *>(&s_f[wid][px][d0]);
+                        const float z8[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
 #pragma unroll
-                        for (int q = 0; q < EPL / 4; ++q) {
-                            const float4 fv = fr[q];
-                            accW[4 * q] = fmaf(zk, fv.x, accW[4 * q]);
-                            accW[4 * q + 1] = fmaf(zk, fv.y, accW[4 * q + 1]);
-                            accW[4 * q + 2] = fmaf(zk, fv.z, accW[4 * q + 2]);
-                            accW[4 * q + 3] = fmaf(zk, fv.w, accW[4 * q + 3]);
+                        for (int k = 0; k < 8; ++k) {
+                            accW[k][0] = fma2(make_float2(z8[k], z8[k]), make_float2(fv.x, fv.y), accW[k][0]);
+                            accW[k][1] = fma2(make_float2(z8[k], z8[k]), make_float2(fv.z, fv.w), accW[k][1]);
                         }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < EPL; ++e) accW[e] = fmaf(zk, s_f[wid][px][d0 + e], accW[e]);
                     }
+                    accb[0] = __fadd2_rn(accb[0], make_float2(za.x, za.y));
+                    accb[1] = __fadd2_rn(accb[1], make_float2(za.z, za.w));
+                    accb[2] = __fadd2_rn(accb[2], make_float2(zb.x, zb.y));
+                    accb[3] = __fadd2_rn(accb[3], make_float2(zb.z, zb.w));
                 }
-                if (lane < KC) accb += s_dz[wid][px][lane];
             }
             __syncwarp();
         }
-    }
-    // the warps' sums enter the block's in warp order (one warp at a time), so the decoder
-    // gradient is the same bits on every run and through every entry point
-    for (int w = 0; w < SH::WARPS; ++w) {
-        if (K > 0 && wid == w) {
-            if constexpr (D > 0) {
-                if (kr < K) {
+        // the gradient of the logits (the factored form; W^T dz is left to the backward) or of the features
+        if (g_coef) {
 #pragma unroll
-                    for (int e = 0; e < EPL; ++e) s_dW[kr * D + d0 + e] += accW[e];
+            for (int p = 0; p < NPX; ++p) {
+                const uint32_t i = base + p * NT + tid;
+#pragma unroll
+                for (int k = 0; k < KC; ++k)
+                    if (k < K && i < n_px) (g_coef + k * P)[i] = dz[p][k];
+            }
+        } else if constexpr (D > 0) {
+            float2 gf[NPX][D / 2];
+#pragma unroll
+            for (int p = 0; p < NPX; ++p)
+#pragma unroll
+                for (int d = 0; d < D / 2; ++d) gf[p][d] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                if (k < K) {
+                    const float4 *wr = reinterpret_cast<const float4 *>(s_W + k * D);
+#pragma unroll
+                    for (int q = 0; q < D / 4; ++q) {
+                        const float4 w4 = wr[q];
+#pragma unroll
+                        for (int p = 0; p < NPX; ++p) {
+                            const float2 z = make_float2(dz[p][k], dz[p][k]);
+                            gf[p][2 * q] = fma2(make_float2(w4.x, w4.y), z, gf[p][2 * q]);
+                            gf[p][2 * q + 1] = fma2(make_float2(w4.z, w4.w), z, gf[p][2 * q + 1]);
+                        }
+                    }
                 }
             }
-            if (lane < K) s_dW[K * D + lane] += accb;
+#pragma unroll
+            for (int p = 0; p < NPX; ++p) {
+                const uint32_t i = base + p * NT + tid;
+                if (i < n_px) {
+    #pragma unroll
+                    for (int d = 0; d < D / 2; ++d) {
+                        (g_feat + 2 * d * P)[i] = gf[p][d].x;
+                        (g_feat + (2 * d + 1) * P)[i] = gf[p][d].y;
+                    }
+                }
+            }
+        }
+    }
+    // the groups' tiles by shuffles, then the warps' in warp order (one warp at a time), so the decoder
+    // gradient is the same bits on every run and through every entry point
+    if (K > 0) {
+#pragma unroll
+        for (int g = 1; g < GROUPS; ++g) {
+            const int src = (lane + g * TILES) & 31;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float x = __shfl_sync(0xffffffffu, accW[k][h].x, src), y = __shfl_sync(0xffffffffu, accW[k][h].y, src);
+                    if (grp == 0) accW[k][h] = __fadd2_rn(accW[k][h], make_float2(x, y));
+                }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float x = __shfl_sync(0xffffffffu, accb[k].x, src), y = __shfl_sync(0xffffffffu, accb[k].y, src);
+                if (grp == 0) accb[k] = __fadd2_rn(accb[k], make_float2(x, y));
+            }
+        }
+    }
+    for (int w = 0; w < SH::WARPS; ++w) {
+        if (K > 0 && wid == w && grp == 0) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (k0 + k >= K) continue;
+                if constexpr (D > 0) {
+                    float *o = s_dW + (k0 + k) * D + d0;
+                    o[0] += accW[k][0].x;
+                    o[1] += accW[k][0].y;
+                    o[2] += accW[k][1].x;
+                    o[3] += accW[k][1].y;
+                }
+                if (d0 == 0) s_dW[K * D + k0 + k] += k % 2 ? accb[k / 2].y : accb[k / 2].x;
+            }
         }
         __syncthreads();
     }
     // per-block partials, weighted and normalised by the view's pixel count
-    const double wc = block_sum_f64((double)lc * lp.color / (double)Pv, s_red);
-    const double wd = block_sum_f64((double)ld * lp.depth / (double)Pv, s_red);
-    const double wsm = block_sum_f64((double)ls * lp.sem / (double)Pv, s_red);
-    __syncthreads();
+    const float x[3] = {lc, ld, ls};
+    double sums[3];
+    block_sums_f64<NT, false>(x, nullptr, sums);
     for (int j = tid; j < nval; j += NT) part_f[(size_t)blk * nval + j] = s_dW[j];
-    if (tid == 0) {
-        part_d[3 * blk] = wc;
-        part_d[3 * blk + 1] = wd;
-        part_d[3 * blk + 2] = wsm;
+    if (tid < 3) {
+        const double w = tid == 0 ? lp.color : tid == 1 ? lp.depth : lp.sem;
+        part_d[3 * blk + tid] = (tid == 0 ? sums[0] : tid == 1 ? sums[1] : sums[2]) * w / (double)Pv;
     }
 }
 
@@ -508,11 +642,12 @@ __global__ void __launch_bounds__(256) dsr_stats_kernel(int64_t m, const float *
         s1.add(s);
         s2.add(s * s);
     });
-    const double t1 = block_sum_f64((double)s1.s - s1.c, s_red);
-    const double t2 = block_sum_f64((double)s2.s - s2.c, s_red);
+    const float x[2] = {s1.s, s2.s}, lo[2] = {s1.c, s2.c};
+    double t[2];
+    block_sums_f64<256, true>(x, lo, t);
     if (threadIdx.x == 0) {
-        part[2 * blockIdx.x] = t1;
-        part[2 * blockIdx.x + 1] = t2;
+        part[2 * blockIdx.x] = t[0];
+        part[2 * blockIdx.x + 1] = t[1];
     }
     if (!last_block(ctr)) return;
     const double u1 = sum_partials_cg(part, 2, 0, gridDim.x, s_red);
@@ -546,8 +681,10 @@ __global__ void __launch_bounds__(256) dsr_mask_kernel(int64_t m, const float *l
         if (s > bd.x) { sb.add(s); ++nb; }
         if (s < bd.y) { ss.add(-l); ++ns; }
     });
-    const double t[4] = {block_sum_f64((double)sb.s - sb.c, s_red), block_sum_f64((double)nb, s_red),
-                         block_sum_f64((double)ss.s - ss.c, s_red), block_sum_f64((double)ns, s_red)};
+    // a thread's counts are far below 2^24: exact in f32
+    const float x[4] = {sb.s, (float)nb, ss.s, (float)ns}, lo[4] = {sb.c, 0.f, ss.c, 0.f};
+    double t[4];
+    block_sums_f64<256, true>(x, lo, t);
     if (threadIdx.x == 0)
         for (int k = 0; k < 4; ++k) mask_part[4 * blockIdx.x + k] = t[k];
     if (!last_block(ctr)) return;
@@ -590,13 +727,14 @@ constexpr int kPoseBlocks = 128;
 __global__ void __launch_bounds__(256) pose_reduce_kernel(int64_t n, const float *pose_part, double *d_twist) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
-    __shared__ double s_red[8];
     const int vk = blockIdx.y;  // view * 6 + component
     const float *p = pose_part + (int64_t)vk * n;
     Kahan s;
     for_my_elements(n, p, [&](int64_t, float x) { s.add(x); });
-    const double t = block_sum_f64((double)s.s - s.c, s_red);
-    if (threadIdx.x == 0 && t != 0) atomicAdd(&d_twist[vk], t);
+    const float x[1] = {s.s}, lo[1] = {s.c};
+    double t[1];
+    block_sums_f64<256, true>(x, lo, t);
+    if (threadIdx.x == 0 && t[0] != 0) atomicAdd(&d_twist[vk], t[0]);
 }
 
 // ------------------------------------------------------------------ pose step
@@ -694,14 +832,30 @@ __global__ void pose_step_kernel(int n_views, const double *grad, double *Tst, d
     }
 }
 
-// Blocks per view: at most one resident wave of the loss kernel over all views (resident
-// = blocks per SM x SMs of the current device; 0 = unknown), and at most kLossBlocks in all.
-int loss_blocks_x(const ViewTable &vt, int resident = 0) {
+// Blocks per view of the median's passes.
+int median_blocks_x(const ViewTable &vt) {
     int64_t maxPv = 0;
     for (int v = 0; v < vt.n_views; ++v) maxPv = std::max<int64_t>(maxPv, (int64_t)vt.W[v] * vt.H[v]);
-    const int total = resident > 0 ? std::min(resident, kLossBlocks) : kLossBlocks;
-    const int per_view = std::max(1, total / vt.n_views);
+    const int per_view = std::max(1, kMedianBlocks / vt.n_views);
     return (int)std::max<int64_t>(1, std::min<int64_t>((maxPv + 255) / 256, per_view));
+}
+
+// The loss kernel's blocks: at most one resident wave (resident = blocks per SM x SMs of the current
+// device; 0 = unknown) and at most kLossBlocks in all, shared among the views in proportion to their
+// pixels (each view at least one), so that views of different sizes finish together: on eight keyframes of
+// 1200x680 and 640x363 in turn, equal shares left the blocks of the small views idle for most of
+// the kernel.
+LossGrid loss_grid(const ViewTable &vt, int resident, int pixels_per_block) {
+    const int64_t P = vt.pix_off[vt.n_views];
+    const int total = std::max(vt.n_views, resident > 0 ? std::min(resident, kLossBlocks) : kLossBlocks);
+    LossGrid g;
+    g.off[0] = 0;
+    for (int v = 0; v < vt.n_views; ++v) {
+        const int64_t Pv = (int64_t)vt.W[v] * vt.H[v];
+        const int64_t share = (int64_t)(total - vt.n_views) * Pv / P + 1;  // the shares' sum is at most total
+        g.off[v + 1] = g.off[v] + (int)std::min<int64_t>(share, (Pv + pixels_per_block - 1) / pixels_per_block);
+    }
+    return g;
 }
 
 template <typename K>
@@ -713,24 +867,36 @@ int resident_blocks(K kernel, int threads) {
     return per_sm * sms;
 }
 
+template <int D, int KC>
+gs_status launch_loss_kernel(const ViewTable &vt, const LossP &lp, const gs_images *img, const gs_targets *tgt,
+                             const float *W, const float *b, int64_t P, const uint32_t *mh, gs_image_grads_out *g,
+                             float *part_f, double *part_d, float *mask_out, float *median_out, cudaStream_t st,
+                             int *rows) {
+    using SH = LossShape<D, KC>;
+    const LossGrid lg = loss_grid(vt, resident_blocks(loss_kernel<D, KC>, SH::NT), SH::NT * SH::NPX);
+    *rows = lg.off[vt.n_views];
+    return launch_pdl(loss_kernel<D, KC>, *rows, SH::NT, 0, st, vt, lg, lp, img->rgb, img->depth, img->sil, img->feat,
+                      tgt->rgb, tgt->depth, tgt->label, W, b, P, mh, g->rgb, g->depth, g->sil, g->feat, g->feat_coef,
+                      part_f, part_d, mask_out, median_out);
+}
+
 template <int D>
 gs_status launch_loss(const ViewTable &vt, const LossP &lp, const gs_images *img, const gs_targets *tgt,
                       const float *W, const float *b, int64_t P, const uint32_t *mh, gs_image_grads_out *g,
                       float *part_f, double *part_d, float *dW, float *db, double *loss_out, float *mask_out,
                       float *median_out, cudaStream_t st) {
-    const int bx = loss_blocks_x(vt, lp.K <= 8 ? resident_blocks(loss_kernel<D, 8>, LossShape<D, 8>::NT)
-                                              : resident_blocks(loss_kernel<D, kMaxK>, LossShape<D, kMaxK>::NT));
-    dim3 grid(bx, vt.n_views);
-    const gs_status ls =
-        lp.K <= 8 ? launch_pdl(loss_kernel<D, 8>, grid, LossShape<D, 8>::NT, 0, st, vt, lp, img->rgb, img->depth,
-                               img->sil, img->feat, tgt->rgb, tgt->depth, tgt->label, W, b, P, mh, g->rgb, g->depth,
-                               g->sil, g->feat, g->feat_coef, part_f, part_d, mask_out, median_out)
-                  : launch_pdl(loss_kernel<D, kMaxK>, grid, LossShape<D, kMaxK>::NT, 0, st, vt, lp, img->rgb,
-                               img->depth, img->sil, img->feat, tgt->rgb, tgt->depth, tgt->label, W, b, P, mh,
-                               g->rgb, g->depth, g->sil, g->feat, g->feat_coef, part_f, part_d, mask_out,
-                               median_out);
+    int rows_f = 0;
+    auto launch = [&](auto kc) {
+        return launch_loss_kernel<D, decltype(kc)::value>(vt, lp, img, tgt, W, b, P, mh, g, part_f, part_d, mask_out,
+                                                          median_out, st, &rows_f);
+    };
+    // the class bound in steps of 8: registers, shared memory and the unrolled work follow it
+    const gs_status ls = lp.K <= 8    ? launch(std::integral_constant<int, 8>())
+                         : lp.K <= 16 ? launch(std::integral_constant<int, 16>())
+                         : lp.K <= 24 ? launch(std::integral_constant<int, 24>())
+                                      : launch(std::integral_constant<int, 32>());
     if (ls) return ls;
-    int rows = bx * vt.n_views;
+    int rows = rows_f;
     if (lp.ssim_coef != 0.f) {
         // the SSIM tiles add their colour-term shares as further partial rows
         const gs_status s = launch_ssim(vt, lp.ssim_coef, img->rgb, tgt->rgb, lp.ssim_maps, part_d + 3 * (size_t)rows,
@@ -738,8 +904,8 @@ gs_status launch_loss(const ViewTable &vt, const LossP &lp, const gs_images *img
         if (s) return s;
         rows += ssim_blocks(vt);
     }
-    return launch_pdl(loss_finish_kernel, lp.K * D + lp.K + 4, 256, 0, st, bx * vt.n_views, rows, lp.K, D, part_f,
-                      part_d, dW, db, loss_out);
+    return launch_pdl(loss_finish_kernel, lp.K * D + lp.K + 4, 256, 0, st, rows_f, rows, lp.K, D, part_f, part_d, dW, db,
+                      loss_out);
 }
 
 }  // namespace
@@ -771,11 +937,7 @@ extern "C" gs_status gs_loss_fwd_bwd(const gs_camera *cams, int n_views, int fea
     const int64_t P = vt.pix_off[n_views];
     gs_status s;
     if (lp->mask_mode == 1) {
-        if ((s = cuda_status(cudaMemsetAsync(mh, 0, sizeof(uint32_t) * 4 * 256 * n_views, st)))) return s;
-        dim3 grid(loss_blocks_x(vt), n_views);
-        for (int pass = 0; pass < 4; ++pass)
-            median_hist_kernel<<<grid, 256, 0, st>>>(vt, pass, img->depth, tgt->depth, mh);
-        if ((s = last_launch())) return s;
+        if ((s = launch_median(vt, img->depth, tgt->depth, mh, median_blocks_x(vt), st))) return s;
     }
     // Eq. 15: the L1 part weighted lambda_c (1 - lambda), the SSIM part lambda_c lambda
     LossP q{lp->color * (1.f - lp->ssim), lp->depth, lp->sem, lp->tau_obs, lp->mask_mode, lp->n_classes,
@@ -955,11 +1117,7 @@ extern "C" gs_status gs_loss_fwd_bwd_noalloc(const gs_camera *cams, int n_views,
     const int64_t P = vt.pix_off[n_views];
     if (lp->mask_mode == 1) {
         // the histograms keep the previous call's counts: clear them first
-        if ((s = cuda_status(cudaMemsetAsync(mh, 0, sizeof(uint32_t) * 4 * 256 * n_views, st)))) return s;
-        dim3 grid(loss_blocks_x(vt), n_views);
-        for (int pass = 0; pass < 4; ++pass)
-            median_hist_kernel<<<grid, 256, 0, st>>>(vt, pass, img->depth, tgt->depth, mh);
-        if ((s = last_launch())) return s;
+        if ((s = launch_median(vt, img->depth, tgt->depth, mh, median_blocks_x(vt), st))) return s;
     }
     LossP q{lp->color, lp->depth, lp->sem, lp->tau_obs, lp->mask_mode, lp->n_classes};
 #define GS_LOSS(DD)                                                                                              \
@@ -1128,10 +1286,7 @@ extern "C" gs_status gs_expand(const gs_camera *cams, int n_views, const gs_imag
     cudaStream_t st = (cudaStream_t)stream;
     gs_status s;
     if ((s = cuda_status(cudaMemsetAsync(status, 0, sizeof(int32_t), st)))) return s;
-    if ((s = cuda_status(cudaMemsetAsync(mh, 0, sizeof(uint32_t) * 4 * 256 * n_views, st)))) return s;
-    const dim3 hgrid(loss_blocks_x(vt), n_views);
-    for (int pass = 0; pass < 4; ++pass)
-        median_hist_kernel<<<hgrid, 256, 0, st>>>(vt, pass, img->depth, tgt->depth, mh);
+    if ((s = launch_median(vt, img->depth, tgt->depth, mh, median_blocks_x(vt), st))) return s;
     const dim3 grid(bx, n_views);
     expand_count_kernel<<<grid, 256, 0, st>>>(vt, img->sil, img->depth, tgt->depth, mh, tau_unobs, counts);
     expand_scan_kernel<<<1, 1024, 0, st>>>(counts, (int64_t)n_views * bx, offsets, n_new);

@@ -128,7 +128,7 @@ typedef struct {
      * about 0.3 s); negative = a block gives up at the first earlier block it
      * looks at (a test hook: gs_bin_sort then reports GS_ERR_TIMEOUT whenever a
      * radix pass has more than one block of keys: 1,024 visible items per depth
-     * pass block up to 2^21 (view, Gaussian) items and 2,048 above, 8,192
+     * pass block up to 2^21 (view, Gaussian) items and 2,048 above, 4,096
      * instances per tile pass block; and a GS_BLOCKS_RING
      * forward whenever one of its warps has to wait for another). */
     int32_t spin_limit;

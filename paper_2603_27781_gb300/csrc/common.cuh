@@ -240,18 +240,19 @@ template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16
 }
 
 // Exact tile rectangle of a splat (half-open, in tiles): floor((u - r)/16) is
-// floordiv(floor(u) - r, 16) because r is an integer.
+// floordiv(floor(u) - r, 16) because r is an integer.  In 32 bits: r is at most 2^24 and an image at most 2^15
+// wide, so a centre beyond 2^26 (and one that is not a number, taken as -2^26) lies on the same side of every
+// tile as 2^26 does.
 __device__ __forceinline__ void tile_rect(float u, float v, int r, int TX, int TY, int &x0, int &y0,
                                           int &x1, int &y1) {
-    const float lim = 1099511627776.0f;  // 2^40
-    float fu = fminf(fmaxf(floorf(u), -lim), lim), fv = fminf(fmaxf(floorf(v), -lim), lim);
-    long long iu = (long long)fu, iv = (long long)fv;
-    auto fdiv = [](long long a) -> long long { return a >= 0 ? a / kTile : -((-a + kTile - 1) / kTile); };
-    auto cl = [](long long a, long long hi) -> int { return (int)(a < 0 ? 0 : (a > hi ? hi : a)); };
-    x0 = cl(fdiv(iu - r), TX);
-    y0 = cl(fdiv(iv - r), TY);
-    x1 = cl(fdiv(iu + r) + 1, TX);
-    y1 = cl(fdiv(iv + r) + 1, TY);
+    const float lim = 67108864.0f;  // 2^26
+    const int iu = (int)fminf(fmaxf(floorf(u), -lim), lim), iv = (int)fminf(fmaxf(floorf(v), -lim), lim);
+    auto cl = [](int a, int hi) { return min(max(a, 0), hi); };
+    static_assert(kTile == 16, "a tile is 2^4 pixels");
+    x0 = cl((iu - r) >> 4, TX);
+    y0 = cl((iv - r) >> 4, TY);
+    x1 = cl(((iu + r) >> 4) + 1, TX);
+    y1 = cl(((iv + r) >> 4) + 1, TY);
 }
 
 // Programmatic dependent launch: a kernel launched with launch_pdl may start (be scheduled,
@@ -357,7 +358,7 @@ constexpr int kSortThreads = 256;       // threads of a depth-sort pass block
 constexpr int64_t kSortSmallItems = (int64_t)1 << 21;
 constexpr int kSortIPTSmall = 4, kSortIPTLarge = 8;  // keys per thread of a depth-sort pass
 inline int depth_sort_tile(int64_t vn) { return kSortThreads * (vn <= kSortSmallItems ? kSortIPTSmall : kSortIPTLarge); }
-constexpr int kSortThreadsInst = 1024;  // threads of a tile-sort pass block
+constexpr int kSortThreadsInst = 512;   // threads of a tile-sort pass block
 constexpr int kSortIPTInst = 8;         // keys per thread of a tile-sort pass
 constexpr int kSortTileInst = kSortThreadsInst * kSortIPTInst;
 constexpr int kScanIPT = 8;

@@ -529,34 +529,50 @@ __global__ void __launch_bounds__(LossShape<D, KC>::NT, LossShape<D, KC>::BLOCKS
 }
 
 // Sums the per-block partials in a fixed order (nblk rows of decoder partials, nrows_d rows
-// of loss-term partials: the loss blocks, then any SSIM tiles).  Block j < K*D+K reduces decoder
-// gradient column j; blocks nval+t (t < 3) loss term t; block nval+3 the total
-// (recomputing the three terms in the same order, so the total is their exact sum).
-__global__ void __launch_bounds__(256) loss_finish_kernel(int nblk, int nrows_d, int K, int D, const float *part_f,
-                                                          const double *part_d, float *dW, float *db,
-                                                          double *loss_out) {
+// of loss-term partials: the loss blocks, then any SSIM tiles).  A warp sums each decoder gradient
+// column (no barrier: the few hundred rows are one round of loads); the last block sums the three loss
+// terms and their total.
+constexpr int kFinishThreads = 256;
+__global__ void __launch_bounds__(kFinishThreads) loss_finish_kernel(int nblk, int nrows_d, int K, int D, const float *part_f,
+                                                                     const double *part_d, float *dW, float *db,
+                                                                     double *loss_out) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
-    __shared__ double s_red[8];
-    const int nval = K * D + K, j = blockIdx.x;
-    if (j < nval) {
+    const int nval = K * D + K, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (blockIdx.x + 1 < gridDim.x) {
+        const int j = blockIdx.x * (kFinishThreads / 32) + w;
+        if (j >= nval) return;
         double x = 0;
-        for (int b = threadIdx.x; b < nblk; b += 256) x += (double)part_f[(size_t)b * nval + j];
-        const double t = block_sum_f64(x, s_red);
-        if (threadIdx.x == 0) {
-            if (j < K * D) dW[j] = (float)t;
-            else db[j - K * D] = (float)t;
+#pragma unroll 8
+        for (int b = lane; b < nblk; b += 32) x += (double)part_f[(size_t)b * nval + j];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) {
+            if (j < K * D) dW[j] = (float)x;
+            else db[j - K * D] = (float)x;
         }
         return;
     }
-    const int term = j - nval;
-    double tot[3];
+    __shared__ double s_red[3][kFinishThreads / 32];
+    double x[3] = {0, 0, 0};
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nrows_d; b += kFinishThreads)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[c] += part_d[3 * (size_t)b + c];
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
-        double x = 0;
-        for (int b = threadIdx.x; b < nrows_d; b += 256) x += part_d[3 * b + c];
-        tot[c] = block_sum_f64(x, s_red);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x[c] += __shfl_xor_sync(0xffffffffu, x[c], o);
+        if (lane == 0) s_red[c][w] = x[c];
     }
-    if (threadIdx.x == 0) loss_out[term < 3 ? 1 + term : 0] = term < 3 ? tot[term] : tot[0] + tot[1] + tot[2];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t[3] = {0, 0, 0};
+        for (int c = 0; c < 3; ++c)
+            for (int i = 0; i < kFinishThreads / 32; ++i) t[c] += s_red[c][i];
+        loss_out[0] = t[0] + t[1] + t[2];
+        for (int c = 0; c < 3; ++c) loss_out[1 + c] = t[c];
+    }
 }
 
 // --------------------------------------------------------------------- DSR
@@ -904,8 +920,8 @@ gs_status launch_loss(const ViewTable &vt, const LossP &lp, const gs_images *img
         if (s) return s;
         rows += ssim_blocks(vt);
     }
-    return launch_pdl(loss_finish_kernel, lp.K * D + lp.K + 4, 256, 0, st, rows_f, rows, lp.K, D, part_f, part_d, dW, db,
-                      loss_out);
+    return launch_pdl(loss_finish_kernel, ceil_div(lp.K * D + lp.K, kFinishThreads / 32) + 1, kFinishThreads, 0, st, rows_f,
+                      rows, lp.K, D, part_f, part_d, dW, db, loss_out);
 }
 
 }  // namespace
@@ -977,7 +993,8 @@ gs_status dsr_grad(int64_t n, const float *log_scales, float lam_big, float lam_
                    float *d_log_scales, cudaStream_t st) {
     if (n == 0) return GS_OK;
     const int64_t m = 3 * n;
-    return launch_pdl(dsr_grad_kernel, std::min(ceil_div(m, 256), kRedBlocks), 256, 0, st, m, log_scales, lam_big,
+    // no partials here: enough blocks for every thread to hold four 16-byte loads at a time
+    return launch_pdl(dsr_grad_kernel, std::min(ceil_div(m, 256 * 16), kSMs * 16), 256, 0, st, m, log_scales, lam_big,
                       lam_small, out, d_log_scales);
 }
 }  // namespace

@@ -13,12 +13,12 @@
 //
 // The digit histograms of every pass are counted by the kernels that write the keys (the
 // compaction for the depth keys, the emission for the tile keys) with shared-memory atomics.
-// Each radix pass is one kernel: a block ranks its keys (1024 or 2048 in a depth pass, 8192 in a tile
-// pass) stably within the block (peer lanes of a digit from match_any + per-warp digit
+// Each radix pass is one kernel: a block ranks its keys (1024 or 2048 in a depth pass, 4096 in a tile
+// pass) stably within the block (peer lanes of a digit from one ballot per digit bit + per-warp digit
 // counters), publishes its per-digit
 // counts, finds its global offsets by a chained look-back over earlier blocks,
-// and scatters through shared memory.  Blocks take tile numbers from an atomic
-// counter so a block only waits on blocks that are already running; every wait
+// and scatters through shared memory.  Blocks take chunks of keys from an atomic
+// counter until none is left, so a block only waits on chunks that a running block has taken; every wait
 // is bounded and reports GS_ERR_TIMEOUT in the status word if it gives up.
 #include <type_traits>
 
@@ -68,45 +68,60 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t *t
     return r;
 }
 
-// ------------------------------------------------------------ state of a call
-// Zeroes what a binning accumulates into: the ranges, the counters, the instance count and
-// status word, the queued forward's work counters, the tile counts, the emission's per-block
-// instance counts, the digit histograms and the look-back flags (the last and largest in 16-byte
-// stores over the whole grid).
-__global__ void __launch_bounds__(256) bin_init_kernel(uint32_t *ranges, int64_t n_ranges, uint32_t *counters,
-                                                       int64_t *n_inst, int32_t *status, uint32_t *tile_counts,
-                                                       int64_t n_tiles, uint32_t *emit_sums, int64_t n_emit,
-                                                       uint32_t *hist, uint4 *lookback, int64_t n_lookback4,
-                                                       uint32_t *queue) {
-    pdl_wait();
-    pdl_trigger();
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t i = i0; i < n_lookback4; i += stride) lookback[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int64_t i = i0; i < n_ranges; i += stride) ranges[i] = 0u;
-    for (int64_t i = i0; i < n_tiles; i += stride) tile_counts[i] = 0u;
-    for (int64_t i = i0; i < n_emit; i += stride) emit_sums[i] = 0u;
-    for (int64_t i = i0; i < 8 * 256; i += stride) hist[i] = 0u;
-    for (int64_t i = i0; i < 64; i += stride) counters[i] = 0u;
-    if (i0 == 0) {
-        *n_inst = 0;
-        *status = 0;
-        if (queue) queue[0] = queue[1] = 0u;
-    }
+// ------------------------------------------------ compaction of visible items
+// Block b looks at items [b kScanBlock, (b + 1) kScanBlock), warp w of it at the 32 kScanIPT items from
+// 32 kScanIPT w on, 32 consecutive ones at a time.
+__device__ __forceinline__ int64_t scan_base() {
+    return (int64_t)blockIdx.x * kScanBlock + (int64_t)(threadIdx.x >> 5) * (32 * kScanIPT) + (threadIdx.x & 31);
 }
 
-// ------------------------------------------------ compaction of visible items
-__global__ void __launch_bounds__(256) vis_reduce_kernel(const int32_t *touched, int64_t count, uint32_t *block_sums) {
+// What a binning accumulates into, zeroed by its first kernel.
+struct BinState {
+    uint32_t *ranges, *counters, *tile_counts, *emit_sums, *hist, *queue;
+    uint4 *lookback;
+    int64_t n_ranges, n_tiles, n_emit, n_lookback4;
+    int64_t *n_inst;
+    int32_t *status;
+};
+
+// First kernel of a binning: zeroes what the call accumulates into (the ranges, the counters, the instance
+// count and status word, the queued forward's work counters, the tile counts, the emission's per-block
+// instance counts, the digit histograms and the look-back flags, the last and largest in 16-byte stores over
+// the whole grid) and counts the visible items of its scan block (grid: at least the count's scan blocks).
+__global__ void __launch_bounds__(256) init_reduce_kernel(BinState b, const int32_t *touched, int64_t count,
+                                                          uint32_t *block_sums) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
-    __shared__ uint32_t s_warp[9];
-    int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanIPT;
+    __shared__ uint32_t s_warp[8];
+    const int64_t base = scan_base();
+    bool f[kScanIPT];
+#pragma unroll
+    for (int k = 0; k < kScanIPT; ++k) f[k] = base + 32 * k < count && touched[base + 32 * k] > 0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t i = i0; i < b.n_lookback4; i += stride) b.lookback[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int64_t i = i0; i < b.n_ranges; i += stride) b.ranges[i] = 0u;
+    for (int64_t i = i0; i < b.n_tiles; i += stride) b.tile_counts[i] = 0u;
+    for (int64_t i = i0; i < b.n_emit; i += stride) b.emit_sums[i] = 0u;
+    for (int64_t i = i0; i < 8 * 256; i += stride) b.hist[i] = 0u;
+    for (int64_t i = i0; i < 64; i += stride) b.counters[i] = 0u;
+    if (i0 == 0) {
+        *b.n_inst = 0;
+        *b.status = 0;
+        if (b.queue) b.queue[0] = b.queue[1] = 0u;
+    }
+    if ((int64_t)blockIdx.x * kScanBlock >= count) return;  // whole block
     uint32_t c = 0;
 #pragma unroll
-    for (int k = 0; k < kScanIPT; ++k) c += (base + k < count && touched[base + k] > 0) ? 1u : 0u;
-    uint32_t tot;
-    block_exclusive_scan(c, &tot, s_warp);
-    if (threadIdx.x == 0) block_sums[blockIdx.x] = tot;
+    for (int k = 0; k < kScanIPT; ++k) c += __popc(__ballot_sync(0xffffffffu, f[k]));
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t tot = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) tot += s_warp[w];
+        block_sums[blockIdx.x] = tot;
+    }
 }
 
 // Single-block exclusive scan of nb block sums; total -> counters[slot].
@@ -118,7 +133,7 @@ __global__ void __launch_bounds__(1024) blocksum_scan_kernel(uint32_t *block_sum
                                                              int64_t capacity, int64_t *n_inst, int32_t *status) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
-    __shared__ uint32_t s_part[1024];
+    __shared__ uint32_t s_warp[33];
     const bool failed = binning_failed(status);
     int64_t nb = nb_from ? ((int64_t)*nb_from + items_per_block - 1) / items_per_block : nb_fixed;
     if (failed) return;  // whole block (the word is only written by earlier kernels)
@@ -126,22 +141,14 @@ __global__ void __launch_bounds__(1024) blocksum_scan_kernel(uint32_t *block_sum
     int64_t b0 = (int64_t)threadIdx.x * per;
     uint32_t s = 0;
     for (int64_t i = b0; i < b0 + per && i < nb; ++i) s += block_sums[i];
-    s_part[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        uint32_t y = threadIdx.x >= o ? s_part[threadIdx.x - o] : 0;
-        __syncthreads();
-        s_part[threadIdx.x] += y;
-        __syncthreads();
-    }
-    uint32_t run = s_part[threadIdx.x] - s;
+    uint32_t total;
+    uint32_t run = block_exclusive_scan<1024>(s, &total, s_warp);
     for (int64_t i = b0; i < b0 + per && i < nb; ++i) {
         uint32_t x = block_sums[i];
         block_sums[i] = run;
         run += x;
     }
-    if (threadIdx.x == 1023) {
-        uint32_t total = s_part[1023];
+    if (threadIdx.x == 0) {
         counters[slot] = total;
         if (cap_slot >= 0) {
             counters[cap_slot] = (int64_t)total > capacity ? (uint32_t)capacity : total;
@@ -151,16 +158,16 @@ __global__ void __launch_bounds__(1024) blocksum_scan_kernel(uint32_t *block_sum
     }
 }
 
-// Adds the 8-bit digits of passes [0, n_passes) of `key` (lanes with `valid`) to the block's
+// Adds the `bits`-wide digits of passes [0, n_passes) of `key` (lanes with `valid`) to the block's
 // shared histograms.  Every lane of the warp calls it.  Per pass: one atomic for the warp
 // when all of its valid lanes have the same digit (the high digits of nearby keys), else one
 // per lane (the low digits, mostly distinct, so the atomics rarely collide).
-__device__ __forceinline__ void hist_add(uint32_t (*sh)[256], int n_passes, bool valid, uint32_t key) {
+__device__ __forceinline__ void hist_add(uint32_t (*sh)[256], int n_passes, int bits, bool valid, uint32_t key) {
     const uint32_t mask = __ballot_sync(0xffffffffu, valid);
     if (!valid) return;
     const int lane = threadIdx.x & 31, first = __ffs(mask) - 1;
     for (int p = 0; p < n_passes; ++p) {
-        const uint32_t d = (key >> (8 * p)) & 255u;
+        const uint32_t d = (key >> (bits * p)) & ((1u << bits) - 1u);
         const uint32_t d0 = __shfl_sync(mask, d, first);
         if (__all_sync(mask, d == d0)) {
             if (lane == first) atomicAdd(&sh[p][d], (uint32_t)__popc(mask));
@@ -188,37 +195,48 @@ __global__ void __launch_bounds__(256) vis_compact_kernel(const int32_t *touched
                                                           uint32_t *hist) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
-    __shared__ uint32_t s_warp[9];
+    __shared__ uint32_t s_warp[8];
     __shared__ uint32_t sh[4][256];
     __shared__ uint32_t s_key[kScanBlock];  // the block's visible keys, in item order
     for (int i = threadIdx.x; i < 4 * 256; i += 256) (&sh[0][0])[i] = 0u;
-    int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanIPT;
+    const int64_t base = scan_base();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     bool f[kScanIPT];
+    uint32_t bal[kScanIPT];
+#pragma unroll
+    for (int k = 0; k < kScanIPT; ++k) f[k] = base + 32 * k < count && touched[base + 32 * k] > 0;
+    uint32_t key[kScanIPT];
+#pragma unroll
+    for (int k = 0; k < kScanIPT; ++k) key[k] = f[k] ? __float_as_uint(uvdo[base + 32 * k].z) : 0u;
+    const uint32_t block_off = block_sums[blockIdx.x];
     uint32_t c = 0;
 #pragma unroll
     for (int k = 0; k < kScanIPT; ++k) {
-        f[k] = base + k < count && touched[base + k] > 0;
-        c += f[k];
+        bal[k] = __ballot_sync(0xffffffffu, f[k]);
+        c += __popc(bal[k]);
     }
-    uint32_t tot;
-    uint32_t loc = block_exclusive_scan(c, &tot, s_warp);
-    uint32_t off = block_sums[blockIdx.x] + loc;
+    if (lane == 0) s_warp[w] = c;
+    __syncthreads();
+    uint32_t loc = 0, tot = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        loc += i < w ? s_warp[i] : 0u;
+        tot += s_warp[i];
+    }
 #pragma unroll
     for (int k = 0; k < kScanIPT; ++k) {
+        const uint32_t at = loc + __popc(bal[k] & lanemask_lt());
         if (f[k]) {
-            const uint32_t key = __float_as_uint(uvdo[base + k].z);
-            keys[off] = key;
-            vals[off] = (uint32_t)(base + k);
-            s_key[loc] = key;
-            ++off;
-            ++loc;
+            keys[block_off + at] = key[k];
+            vals[block_off + at] = (uint32_t)(base + 32 * k);
+            s_key[at] = key[k];
         }
+        loc += __popc(bal[k]);
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
     for (uint32_t i0 = threadIdx.x - lane; i0 < tot; i0 += 256) {  // warp-uniform rounds
         const uint32_t i = i0 + lane;
-        hist_add(sh, 4, i < tot, i < tot ? s_key[i] : 0u);
+        hist_add(sh, 4, 8, i < tot, i < tot ? s_key[i] : 0u);
     }
     hist_flush(sh, 4, hist);
 }
@@ -227,24 +245,25 @@ __global__ void __launch_bounds__(256) vis_compact_kernel(const int32_t *touched
 constexpr int kEmitBlock = 256;  // sorted items per block of the emission kernels
 
 // One thread per sorted item computes its instance offset; the block's instances are then
-// split evenly over its warps, 32 consecutive instances per warp round, each lane finding
-// the item that owns its instance by a binary search over the block's item offsets in
-// shared memory.  Every store is coalesced, and a few long items (large splats) no longer
-// keep one warp of the block busy while the others idle.
+// split evenly over its warps, 32 consecutive instances per warp round.  A round knows the item that
+// owns its first instance; the next 32 items' offsets say at which lanes the following ones begin, so
+// one shared-memory read and one reduction give every lane its owner (a binary search per lane took
+// eight dependent reads).  Every store is coalesced, and a few long items (large splats) do not
+// keep one warp of the block busy while the others idle.  The grid is bounded and its blocks
+// stride over the sorted items, so a batch whose items are mostly out of view launches no blocks for them.
 // Also the digit histograms of the tile sort's n_passes passes over the written keys.
 __global__ void __launch_bounds__(kEmitBlock) emit_kernel(ViewTable vt, const uint32_t *sorted_items,
                                                           const int32_t *touched, const float4 *uvdo,
                                                           const float4 *conic, const uint32_t *counters,
                                                           const uint32_t *block_sums, int64_t capacity,
                                                           uint32_t *tile_keys, uint32_t *inst_vals, int n_passes,
-                                                          uint32_t *hist, int64_t vn, const int32_t *status) {
+                                                          int bits, uint32_t *hist, int64_t vn, const int32_t *status) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
     __shared__ uint32_t s_warp[9];
     __shared__ uint32_t sh[4][256];
-    __shared__ uint32_t s_off[kEmitBlock];   // exclusive instance offset of each item in the block
-    __shared__ uint32_t s_item[kEmitBlock];
-    __shared__ uint4 s_rect[kEmitBlock];     // (x0, y0, width, tiles per row | first tile of the view << 16)
+    __shared__ uint32_t s_off[kEmitBlock];  // exclusive instance offset of each item in the block
+    __shared__ uint4 s_rect[kEmitBlock];    // (first tile, width, tiles per row, item)
     // whole block (the word is only written by earlier kernels): after a failed depth sort or an
     // overflow nothing is emitted
     const bool failed = binning_failed(status);
@@ -252,60 +271,64 @@ __global__ void __launch_bounds__(kEmitBlock) emit_kernel(ViewTable vt, const ui
     if (failed || (int64_t)blockIdx.x * kEmitBlock >= count) return;  // whole block: no barrier is skipped
     for (int i = threadIdx.x; i < 4 * 256; i += kEmitBlock) (&sh[0][0])[i] = 0u;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * kEmitBlock + threadIdx.x;
-    uint32_t item = 0, c = 0;
-    int x0 = 0, y0 = 0, w = 1, tx = 1;
-    uint32_t tb = 0;
-    if (i < count && sorted_items[i] < vn) {
-        item = sorted_items[i];
-        c = (uint32_t)touched[item];
-        const int v = (int)(item / (uint32_t)vt.n);
-        const float4 rec = uvdo[item];
-        int x1, y1;
-        tile_rect(rec.x, rec.y, (int)conic[item].w, vt.TX[v], vt.TY[v], x0, y0, x1, y1);
-        w = max(x1 - x0, 1);
-        tx = vt.TX[v];
-        tb = (uint32_t)vt.tile_off[v];
-    }
-    uint32_t tot;
-    const uint32_t excl = block_exclusive_scan(c, &tot, s_warp);
-    s_off[threadIdx.x] = excl;
-    s_item[threadIdx.x] = item;
-    s_rect[threadIdx.x] = make_uint4((uint32_t)x0, (uint32_t)y0, (uint32_t)w, (uint32_t)tx);
-    if (threadIdx.x == 0) s_warp[8] = tot;
-    __shared__ uint32_t s_tb[kEmitBlock];
-    s_tb[threadIdx.x] = tb;
-    __syncthreads();
-    const uint32_t bbase = block_sums[blockIdx.x];
-    // warp wid takes instances [q_lo, q_hi) of the block, in whole rounds of 32
-    const uint32_t per = ((tot + 32u * (kEmitBlock / 32) - 1) / (32u * (kEmitBlock / 32))) * 32u;
-    const uint32_t q_lo = min(tot, (uint32_t)wid * per), q_hi = min(tot, q_lo + per);
-    for (uint32_t q0 = q_lo; q0 < q_hi; q0 += 32) {
-        const uint32_t q = q0 + lane;
-        const bool valid = q < q_hi;
-        // the owner: the last item whose offset is <= q (items with no instances share offsets)
-        int owner = 0;
+    for (int64_t blk = blockIdx.x; blk * kEmitBlock < count; blk += gridDim.x) {
+        const int64_t i = blk * kEmitBlock + threadIdx.x;
+        uint32_t item = 0, c = 0, first = 0, w = 1, tx = 1;
+        if (i < count && sorted_items[i] < vn) {
+            item = sorted_items[i];
+            c = (uint32_t)touched[item];
+            const int v = (int)(item / (uint32_t)vt.n);
+            const float4 rec = uvdo[item];
+            int x0, y0, x1, y1;
+            tile_rect(rec.x, rec.y, (int)conic[item].w, vt.TX[v], vt.TY[v], x0, y0, x1, y1);
+            w = (uint32_t)max(x1 - x0, 1);
+            tx = (uint32_t)vt.TX[v];
+            first = (uint32_t)vt.tile_off[v] + (uint32_t)y0 * tx + (uint32_t)x0;
+        }
+        const uint32_t bbase = block_sums[blk];
+        uint32_t tot;
+        const uint32_t excl = block_exclusive_scan(c, &tot, s_warp);
+        s_off[threadIdx.x] = excl;
+        s_rect[threadIdx.x] = make_uint4(first, w, tx, item);
+        __syncthreads();
+        // warp wid takes instances [q_lo, q_hi) of the block, in whole rounds of 32
+        const uint32_t per = ((tot + 32u * (kEmitBlock / 32) - 1) / (32u * (kEmitBlock / 32))) * 32u;
+        const uint32_t q_lo = min(tot, (uint32_t)wid * per), q_hi = min(tot, q_lo + per);
+        // the owner of the warp's first instance: the last item whose offset is <= q_lo
+        int own = 0;
 #pragma unroll
         for (int step = kEmitBlock / 2; step >= 1; step >>= 1)
-            if (s_off[owner + step] <= q) owner += step;
-        const int64_t off = (int64_t)bbase + q;
-        const bool write = valid && off < capacity;
-        uint32_t key = 0u;
-        if (write) {
-            const uint4 rc = s_rect[owner];
-            const int k = (int)(q - s_off[owner]);
-            const int ky = k / (int)rc.z, kx = k - ky * (int)rc.z;
-            key = s_tb[owner] + (uint32_t)(((int)rc.y + ky) * (int)rc.w + (int)rc.x + kx);
-            tile_keys[off] = key;
-            inst_vals[off] = s_item[owner];
+            if (s_off[own + step] <= q_lo) own += step;
+        for (uint32_t q0 = q_lo; q0 < q_hi; q0 += 32) {
+            const uint32_t q = q0 + lane;
+            // bit b: an item after `own` begins at instance q0 + b (every sorted item has instances)
+            const int nx = own + 1 + lane;
+            const uint32_t at = nx < kEmitBlock ? s_off[nx] - q0 : 32u;
+            const uint32_t begins = __reduce_or_sync(0xffffffffu, at < 32u ? 1u << at : 0u);
+            const int owner = min(own + __popc(begins & ((2u << lane) - 1u)), kEmitBlock - 1);
+            own = min(own + __popc(begins), kEmitBlock - 1);
+            const int64_t off = (int64_t)bbase + q;
+            const bool write = q < q_hi && off < capacity;
+            uint32_t key = 0u;
+            if (write) {
+                const uint4 rc = s_rect[owner];
+                const uint32_t k = q - s_off[owner];
+                // row of instance k: floor(k / width), by a reciprocal where its rounding (4e-7 relative)
+                // cannot reach the half instance that (k + 1/2) / width is away from a whole number
+                const uint32_t ky = k < (1u << 20) ? (uint32_t)(((float)k + 0.5f) * __fdividef(1.f, (float)rc.y)) : k / rc.y;
+                key = rc.x + ky * rc.z + (k - ky * rc.y);
+                tile_keys[off] = key;
+                inst_vals[off] = rc.w;
+            }
+            hist_add(sh, n_passes, bits, write, key);
         }
-        hist_add(sh, n_passes, write, key);
+        __syncthreads();  // the block's offsets and rectangles are read before the next items' are written
     }
     hist_flush(sh, n_passes, hist);
 }
 
 // ------------------------------------------------------------------ radix sort
-// Shared memory of a radix-pass block of NT threads with IPT keys each (dynamic: 99 KB for 1024 x 8).
+// Shared memory of a radix-pass block of NT threads with IPT keys each (dynamic: 51 KB for 512 x 8).
 template <int NT, int IPT>
 struct SortSmem {
     uint32_t keys[NT * IPT];
@@ -314,24 +337,38 @@ struct SortSmem {
     uint32_t excl[256];   // block-local exclusive digit offsets
     uint32_t glob[256];   // global destination of the digit's first key in this block
     uint32_t dbase[256];  // global exclusive digit base of the pass
-    uint32_t warp[NT / 32 + 1];
+    uint32_t warp[2][8];
     uint32_t tile;
     int failed;
 };
 
-// One radix pass, NT threads per block and IPT keys per thread: 256 threads for the depth
-// passes over the visible items, 1024 for the tile passes over the instances, where a quarter
-// as many blocks means a sixteenth of the look-back's reads (every block starts at once and
-// reads back through about half of the blocks before it).
+// One radix pass over BITS-wide digits, NT threads per block and IPT keys per thread: 256 threads for the
+// depth passes over the visible items, 512 with 8 keys for the tile passes over the instances.
 // Resident blocks per SM the register allocation must allow: four depth-pass blocks of 8 keys a
-// thread (64 registers), six of 4 (40); two tile-pass blocks (32 registers, about 100 bytes
-// spilled, which costs less than a second wave of blocks: tile sort 0.179 -> 0.172 ms on 2.2 M
-// instances).
+// thread (64 registers), six of 4 (40); three tile-pass blocks (42 registers).  Whole binning in ms with
+// tile-pass blocks of 512 x 8 keys at three per SM, 1024 x 8 at two, 512 x 16 at two, 256 x 16 at four: 0.143 / 0.149 /
+// 0.146 / 0.149 (1M Gaussians at 1200x680, 1.7M instances), 0.091 / 0.098 / 0.096 / 0.096 (300k at 811x607),
+// 0.87 / 0.91 / 0.86 / 0.85 (2M, eight keyframes, 22M instances).
 template <int NT, int IPT> constexpr int sort_min_blocks() {
     return NT == 256 ? (IPT >= 8 ? 4 : 6) : (NT == 512 ? 3 : 2);
 }
 
-template <int NT, int IPT>
+// Lanes of the warp with the same digit (among the lanes in `valid`), by one ballot per bit: a fraction of the
+// time of match.any, which takes the distinct values one after another (the ranking of a depth pass's 1,024
+// keys took 2.2 of the block's 8.7 us with it, and takes 0.8).
+template <int BITS>
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d, uint32_t valid) {
+    uint32_t peers = valid;
+#pragma unroll
+    for (int b = 0; b < BITS; ++b) {
+        const bool set = (d >> b) & 1u;
+        const uint32_t m = __ballot_sync(0xffffffffu, set);
+        peers &= set ? m : ~m;
+    }
+    return peers;
+}
+
+template <int NT, int IPT, int BITS>
 __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kernel(const uint32_t *keys_in, const uint32_t *vals_in,
                                                       uint32_t *keys_out, uint32_t *vals_out,
                                                       const uint32_t *count_ptr, int shift,
@@ -342,63 +379,70 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
                                                       uint32_t emit_vn) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
-    constexpr int W = NT / 32, TILE = NT * IPT;
-    static_assert(NT >= 256, "one thread per digit");
+    constexpr int W = NT / 32, TILE = NT * IPT, BINS = 1 << BITS;
+    static_assert(NT >= BINS && BINS >= 32 && BITS <= 8, "one thread per digit");
     extern __shared__ __align__(16) unsigned char sort_smem[];
     SortSmem<NT, IPT> &S = *reinterpret_cast<SortSmem<NT, IPT> *>(sort_smem);
     uint32_t *s_keys = S.keys, *s_vals = S.vals, *s_excl = S.excl, *s_glob = S.glob, *s_dbase = S.dbase;
     uint32_t(*s_whist)[256] = S.whist;
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    // chunks of TILE keys until none is left: a chunk's number comes from the counter, so every chunk
+    // before it has been taken by a block that runs (or has run)
+    for (;;) {
+    __syncthreads();  // the previous chunk's reads of shared memory are done
     if (tid == 0) {
         S.tile = atomicAdd(tile_ctr, 1u);
         S.failed = binning_failed(status);
     }
-    for (int i = tid; i < W * 256; i += NT) (&s_whist[0][0])[i] = 0;
+    for (int i = tid; i < W * BINS; i += NT) s_whist[i / BINS][i % BINS] = 0;
     __syncthreads();
     const uint32_t tile = S.tile;
+    const uint32_t n = *count_ptr;  // below 2^30
+    if ((uint64_t)tile * TILE >= n) return;
+    const uint32_t base = tile * TILE;
     if (S.failed) {
         // an earlier wait gave up (or the count overflowed): this pass's output is not used.  The
         // block still publishes an inclusive prefix (0: never more than the true one, so a block
         // that adds it scatters in bounds) so that no running block waits for it.
-        if (tid < 256) st_relaxed(lookback + (size_t)tile * 256 + tid, kFlagPre);
+        if (tid < BINS) st_relaxed(lookback + (size_t)tile * 256 + tid, kFlagPre);
         return;
     }
-    const int64_t n = *count_ptr;
-    const int64_t base = (int64_t)tile * TILE;
-    if (base >= n) return;
 
-    uint32_t key[IPT], val[IPT], rank[IPT];
+    const uint32_t mine = base + (uint32_t)w * (IPT * 32) + lane;  // this thread's keys: mine + 32 r
+    uint32_t key[IPT], val[IPT], rank2[IPT / 2];  // ranks below TILE <= 2^16, two to a register
+    static_assert(TILE <= 1 << 16 && IPT % 2 == 0, "16-bit ranks");
 #pragma unroll
     for (int r = 0; r < IPT; ++r) {
-        const int64_t i = base + (int64_t)w * (IPT * 32) + r * 32 + lane;
-        key[r] = i < n ? keys_in[i] : 0u;
-        val[r] = i < n ? vals_in[i] : 0u;
+        const bool valid = mine + 32 * r < n;
+        key[r] = valid ? keys_in[mine + 32 * r] : 0u;
+        val[r] = valid ? vals_in[mine + 32 * r] : 0u;
     }
 #pragma unroll
     for (int r = 0; r < IPT; ++r) {
-        const bool valid = base + (int64_t)w * (IPT * 32) + r * 32 + lane < n;
-        const uint32_t d = (key[r] >> shift) & 255u;
-        // lanes with the same digit; an invalid lane matches only itself
-        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? d : 256u + lane);
-        int leader = __ffs(peers) - 1;
-        uint32_t b = 0;
-        if (valid && lane == leader) {
-            b = s_whist[w][d];
-            s_whist[w][d] = b + __popc(peers);
-        }
-        b = __shfl_sync(0xffffffffu, b, leader);
-        rank[r] = b + __popc(peers & lanemask_lt());
+        const bool valid = mine + 32 * r < n;
+        const uint32_t d = (key[r] >> shift) & (BINS - 1u);
+        const uint32_t peers = digit_peers<BITS>(d, __ballot_sync(0xffffffffu, valid));
+        // every lane reads its digit's count so far; the last lane of the digit adds the round's
+        const uint32_t b = s_whist[w][d];
+        const uint32_t rank = b + __popc(peers & lanemask_lt());
+        if (r % 2) rank2[r / 2] |= rank << 16;
+        else rank2[r / 2] = rank;
+        __syncwarp();
+        if (valid && (peers >> lane) == 1u) s_whist[w][d] = b + __popc(peers);
         __syncwarp();
     }
     __syncthreads();
 
-    // per-digit (thread d < 256): warp-exclusive offsets and the block's count, published at once
-    // for later tiles
+    // per-digit (thread d < BINS): warp-exclusive offsets and the block's count, published at once
+    // for later chunks; then the block-exclusive digit offsets and the pass's digit bases, two scans over the
+    // digits that share their barriers
     const int d = tid;
     uint32_t cnt = 0, hist_d = 0;
-    uint32_t *my = lookback + (size_t)tile * 256 + (d & 255);
-    if (d < 256) {
+    uint32_t *my = lookback + (size_t)tile * 256 + (d & (BINS - 1));
+    uint32_t ci = 0, hi = 0;
+    if (d < BINS) {
+        hist_d = pass_hist[d];
 #pragma unroll
         for (int ww = 0; ww < W; ++ww) {
             uint32_t c = s_whist[ww][d];
@@ -406,23 +450,38 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
             cnt += c;
         }
         st_relaxed(my, (tile == 0 ? kFlagPre : kFlagAgg) | cnt);
-        hist_d = pass_hist[d];
+        ci = cnt;
+        hi = hist_d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, ci, o), y = __shfl_up_sync(0xffffffffu, hi, o);
+            if (lane >= o) {
+                ci += x;
+                hi += y;
+            }
+        }
+        if (lane == 31) {
+            S.warp[0][w] = ci;
+            S.warp[1][w] = hi;
+        }
     }
-    // block-exclusive digit offsets and the pass's digit bases
-    uint32_t lb_tot;
-    const uint32_t ex = block_exclusive_scan<NT>(cnt, &lb_tot, S.warp);
-    if (d < 256) s_excl[d] = ex;
-    uint32_t hist_tot;
-    const uint32_t db = block_exclusive_scan<NT>(hist_d, &hist_tot, S.warp);  // its barriers publish s_excl
-    if (d < 256) s_dbase[d] = db;
+    __syncthreads();
+    if (d < BINS) {
+        for (int ww = 0; ww < w; ++ww) {
+            ci += S.warp[0][ww];
+            hi += S.warp[1][ww];
+        }
+        s_excl[d] = ci - cnt;
+        s_dbase[d] = hi - hist_d;
+    }
+    __syncthreads();
 
     // local scatter by digit into shared memory (the keys leave the registers before the wait)
 #pragma unroll
     for (int r = 0; r < IPT; ++r) {
-        int64_t i = base + (int64_t)w * (IPT * 32) + r * 32 + lane;
-        if (i < n) {
-            uint32_t dd = (key[r] >> shift) & 255u;
-            uint32_t pos = s_excl[dd] + s_whist[w][dd] + rank[r];
+        if (mine + 32 * r < n) {
+            const uint32_t dd = (key[r] >> shift) & (BINS - 1u);
+            const uint32_t pos = s_excl[dd] + s_whist[w][dd] + (r % 2 ? rank2[r / 2] >> 16 : rank2[r / 2] & 0xffffu);
             s_keys[pos] = key[r];
             s_vals[pos] = val[r];
         }
@@ -432,9 +491,9 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
     // (all tiles start together, so the chain is as long as the tile number over kWin); spin
     // (bounded) only on a tile that has not published its count yet
     uint32_t prefix = 0;
-    if (tile != 0 && d < 256) {
+    if (tile != 0 && d < BINS) {
         constexpr int kWin = 8;
-        int64_t t = (int64_t)tile - 1;
+        int t = (int)tile - 1;
         bool done = false, timeout = false;
         while (!done && t >= 0) {
             uint32_t w[kWin];
@@ -470,18 +529,18 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
         if (timeout) set_status(status, GS_ERR_TIMEOUT);
         st_relaxed(my, kFlagPre | (prefix + cnt));
     }
-    if (d < 256) s_glob[d] = s_dbase[d] + prefix;
+    if (d < BINS) s_glob[d] = s_dbase[d] + prefix;
     __syncthreads();
 
     // coalesced-by-run global writes, in warp-uniform rounds of 32 consecutive keys
-    const int tile_n = (int)min((int64_t)TILE, n - base);
+    const int tile_n = (int)min((uint32_t)TILE, n - base);
     for (int i0 = tid - lane; i0 < tile_n; i0 += NT) {
         const int i = i0 + lane;
         const bool ok = i < tile_n;
         uint32_t dst = 0u, v = 0u;
         if (ok) {
             const uint32_t k = s_keys[i];
-            const uint32_t dd = (k >> shift) & 255u;
+            const uint32_t dd = (k >> shift) & (BINS - 1u);
             dst = s_glob[dd] + (uint32_t)i - s_excl[dd];
             v = s_vals[i];
             keys_out[dst] = k;
@@ -510,6 +569,7 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
             if (ok && (lane == 31 || s_next != seg) && c) atomicAdd(&emit_sums[seg], c);
         }
     }
+    }
 }
 
 // The optional 64-bit keys (tile << 32 | depth bits) of the sorted instances.  Tile ids and
@@ -532,12 +592,14 @@ struct SortBufs {
     uint32_t *k0, *v0, *k1, *v1;
 };
 
-// Stable LSD sort of (key, val) pairs by `n_passes` 8-bit digits from bit 0, given the
+// Stable LSD sort of (key, val) pairs by `n_passes` digits of BITS bits from bit 0, given the
 // digit histograms of every pass (hist [n_passes][256], written by the kernel that
 // produced the keys).  Input in (k0, v0); output lands in (k0, v0) if n_passes is even,
 // else (k1, v1).  The last pass also adds the tile runs to tile_counts and, with emit_sums,
 // emit_touched[val] to the count of its kEmitBlock-item block of the output (either optional).
-template <int NT, int IPT>
+// The grid is at most one resident wave, whose blocks take chunks until none is left: max_count is the
+// most there can be (every item, the capacity), often several times what there is.
+template <int NT, int IPT, int BITS>
 gs_status radix_sort(SortBufs b, const uint32_t *count_ptr, int64_t max_count, int n_passes, const uint32_t *hist,
                      uint32_t *lookback, int lb_tiles, uint32_t *tile_ctrs, int32_t *status, int spin_limit,
                      cudaStream_t st, uint32_t *tile_counts = nullptr, uint32_t n_tiles = 0,
@@ -550,18 +612,18 @@ gs_status radix_sort(SortBufs b, const uint32_t *count_ptr, int64_t max_count, i
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return GS_ERR_CUDA;
         if (dev < 0 || dev >= 64 || !opted[dev]) {
-            if (cudaFuncSetAttribute(onesweep_kernel<NT, IPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-                cudaSuccess)
+            if (cudaFuncSetAttribute(onesweep_kernel<NT, IPT, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem) != cudaSuccess)
                 return GS_ERR_CUDA;
             if (dev >= 0 && dev < 64) opted[dev] = true;
         }
     }
-    int grid = ceil_div(max_count, (int64_t)NT * IPT);
+    const int grid = std::min(ceil_div(max_count, (int64_t)NT * IPT), kSMs * sort_min_blocks<NT, IPT>());
     uint32_t *ki = b.k0, *vi = b.v0, *ko = b.k1, *vo = b.v1;
     for (int p = 0; p < n_passes; ++p) {
-        const gs_status s = launch_pdl(onesweep_kernel<NT, IPT>, grid, NT, smem, st, ki, vi, ko, vo, count_ptr, 8 * p,
-                                       hist + 256 * p, tile_ctrs + p, lookback + (size_t)p * lb_tiles * 256, status,
-                                       spin_limit, p == n_passes - 1 ? tile_counts : nullptr, n_tiles, emit_touched,
+        const gs_status s = launch_pdl(onesweep_kernel<NT, IPT, BITS>, grid, NT, smem, st, ki, vi, ko, vo, count_ptr,
+                                       BITS * p, hist + 256 * p, tile_ctrs + p, lookback + (size_t)p * lb_tiles * 256,
+                                       status, spin_limit, p == n_passes - 1 ? tile_counts : nullptr, n_tiles, emit_touched,
                                        p == n_passes - 1 ? emit_sums : nullptr, emit_vn);
         if (s) return s;
         uint32_t *tk = ki, *tv = vi;
@@ -589,31 +651,9 @@ __device__ __forceinline__ int order_bucket(uint32_t c) {
     return c < 1024u ? (int)(c >> 2) : (int)min(256u + ((c - 1024u) >> 6), 1023u);
 }
 
-// Exclusive scan of one value per thread over the 1024-thread block; returns the prefix.
-__device__ __forceinline__ uint32_t scan1024(uint32_t x, uint32_t *warp_tot) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t inc = x;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += y;
-    }
-    if (lane == 31) warp_tot[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        const uint32_t t = warp_tot[lane];
-        uint32_t ti = t;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, ti, d);
-            if (lane >= d) ti += y;
-        }
-        warp_tot[lane] = ti - t;  // exclusive over warps
-    }
-    __syncthreads();
-    const uint32_t r = warp_tot[wid] + inc - x;
-    __syncthreads();
-    return r;
+// Exclusive scan of one value per thread over the 1024-thread block; returns the prefix and the total.
+__device__ __forceinline__ uint32_t scan1024(uint32_t x, uint32_t *total, uint32_t *s_warp) {
+    return block_exclusive_scan<1024>(x, total, s_warp);
 }
 
 __global__ void __launch_bounds__(1024) ranges_order_kernel(const uint32_t *counts, int n_tiles, uint32_t *ranges,
@@ -621,28 +661,33 @@ __global__ void __launch_bounds__(1024) ranges_order_kernel(const uint32_t *coun
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
     __shared__ uint32_t hist[1024];
-    __shared__ uint32_t warp_tot[32];
+    __shared__ uint32_t warp_tot[33];
     const int tid = threadIdx.x;
     const bool failed = binning_failed(status);
-    const int per = (n_tiles + 1023) / 1024, t0 = tid * per, t1 = min(n_tiles, t0 + per);
-    uint32_t sum = 0;
-    for (int t = t0; t < t1; ++t) sum += failed ? 0u : counts[t];
-    uint32_t run = scan1024(sum, warp_tot);
-    if (!failed)
-        for (int t = t0; t < t1; ++t) {
-            const uint32_t c = counts[t];
-            ranges[2 * t] = c ? run : 0u;  // empty tiles: [0, 0)
-            ranges[2 * t + 1] = c ? run + c : 0u;
-            run += c;
-        }
-    if (!order) return;  // whole block
     hist[tid] = 0u;
     __syncthreads();
-    for (int t = tid; t < n_tiles; t += 1024) atomicAdd(&hist[order_bucket(failed ? 0u : counts[t])], 1u);
+    // 1,024 consecutive tiles at a time (coalesced), with the running total carried from one to the next
+    uint32_t carry = 0u;
+    for (int t0 = 0; t0 < n_tiles; t0 += 1024) {
+        const int t = t0 + tid;
+        const uint32_t c = t < n_tiles && !failed ? counts[t] : 0u;
+        uint32_t total;
+        const uint32_t run = carry + scan1024(c, &total, warp_tot);
+        if (t < n_tiles) {
+            if (!failed) {
+                ranges[2 * t] = c ? run : 0u;  // empty tiles: [0, 0)
+                ranges[2 * t + 1] = c ? run + c : 0u;
+            }
+            if (order) atomicAdd(&hist[order_bucket(c)], 1u);
+        }
+        carry += total;
+    }
+    if (!order) return;  // whole block
     __syncthreads();
     // exclusive scan over buckets from the highest down: thread i takes bucket 1023 - i
     const uint32_t h = hist[1023 - tid];
-    const uint32_t before = scan1024(h, warp_tot);
+    uint32_t all;
+    const uint32_t before = scan1024(h, &all, warp_tot);
     hist[1023 - tid] = before;  // first slot of bucket 1023 - tid
     __syncthreads();
     for (int t = tid; t < n_tiles; t += 1024) {
@@ -689,12 +734,13 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     // scheduled while its predecessor drains and waits for it (pdl_wait) before reading.
     gs_status s;
     const int64_t n_lb4 = vn > 0 ? 64 * ((int64_t)4 * L.lb_tiles_depth + (int64_t)3 * L.lb_tiles_inst) : 0;
-    const int init_grid = (int)std::max<int64_t>(1, std::min<int64_t>((n_lb4 + 255) / 256, 1216));
     const int64_t nbe = ceil_div(vn, kEmitBlock);  // emission blocks
-    if ((s = launch_pdl(bin_init_kernel, init_grid, 256, 0, st, out->ranges, 2 * total_tiles, counters, out->n_inst,
-                        out->status, tile_counts, total_tiles, emit_sums, nbe + 1, hist,
-                        reinterpret_cast<uint4 *>(lookback), n_lb4, out->queue)))
-        return s;
+    const int nb = ceil_div(vn, kScanBlock);       // scan blocks
+    const int init_grid = std::max<int>({1, nb, (int)std::min<int64_t>((n_lb4 + 255) / 256, kSMs * 8)});
+    const BinState state{out->ranges, counters, tile_counts, emit_sums, hist, out->queue, reinterpret_cast<uint4 *>(lookback),
+                         2 * total_tiles, total_tiles, nbe + 1, n_lb4, out->n_inst, out->status};
+    // 1. the call's state; the visible items of every scan block
+    if ((s = launch_pdl(init_reduce_kernel, init_grid, 256, 0, st, state, proj->tiles_touched, vn, block_sums))) return s;
     if (vn == 0) return write_ranges_order(tile_counts, out, total_tiles, st);
 
     const float4 *uvdo = reinterpret_cast<const float4 *>(proj->uvdo);
@@ -702,9 +748,7 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     uint32_t *dk_a = reinterpret_cast<uint32_t *>(w + L.dkeys_a), *dv_a = reinterpret_cast<uint32_t *>(w + L.dvals_a);
     uint32_t *dk_b = reinterpret_cast<uint32_t *>(w + L.dkeys_b), *dv_b = reinterpret_cast<uint32_t *>(w + L.dvals_b);
 
-    // 1. compact visible items in index order, keyed by depth bits
-    int nb = ceil_div(vn, kScanBlock);
-    if ((s = launch_pdl(vis_reduce_kernel, nb, 256, 0, st, proj->tiles_touched, vn, block_sums))) return s;
+    // compact visible items in index order, keyed by depth bits
     if ((s = launch_pdl(blocksum_scan_kernel, 1, 1024, 0, st, block_sums, nullptr, (int64_t)nb, kScanBlock, counters,
                         (int)CTR_NVIS, -1, (int64_t)0, nullptr, nullptr)))
         return s;
@@ -715,7 +759,7 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     // 2. stable sort of the visible items by depth (4 passes: result in dk_a/dv_a); the last pass
     //    also counts the instances of every emission block of the sorted items
     auto depth_sort = [&](auto ipt) {
-        return radix_sort<kSortThreads, decltype(ipt)::value>(
+        return radix_sort<kSortThreads, decltype(ipt)::value, 8>(
             {dk_a, dv_a, dk_b, dv_b}, counters + CTR_NVIS, vn, 4, hist, lookback, L.lb_tiles_depth, counters + CTR_TILE,
             out->status, prm.spin_limit, st, nullptr, 0, proj->tiles_touched, emit_sums, (uint32_t)vn);
     };
@@ -727,7 +771,11 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     // 3. emit instances in depth order; instance count -> n_inst (clamped copy for the sort)
     int tile_bits = 1;
     while (((int64_t)1 << tile_bits) < total_tiles) ++tile_bits;
-    int tile_passes = (tile_bits + 7) / 8;
+    // the fewest passes of at most 8 bits, and digits no wider than those passes need: fewer digits mean
+    // fewer ballots, counters and look-back words per block and longer runs to write (1200x680: two passes
+    // of 6 bits)
+    const int tile_passes = (tile_bits + 7) / 8;
+    const int digit_bits = std::max(5, (tile_bits + tile_passes - 1) / tile_passes);
     uint32_t *tk_a = reinterpret_cast<uint32_t *>(w + L.tkeys_a), *tk_b = reinterpret_cast<uint32_t *>(w + L.tkeys_b);
     uint32_t *tv_b = reinterpret_cast<uint32_t *>(w + L.tvals_b);
     // the emitted values go where the final pass must not land: out->vals ends the sort
@@ -736,17 +784,24 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     if ((s = launch_pdl(blocksum_scan_kernel, 1, 1024, 0, st, emit_sums, counters + CTR_NVIS, (int64_t)0, kEmitBlock,
                         counters, (int)CTR_MRAW, (int)CTR_M, out->capacity, out->n_inst, out->status)))
         return s;
-    if ((s = launch_pdl(emit_kernel, (int)nbe, kEmitBlock, 0, st, vt, sorted_items, proj->tiles_touched, uvdo, conic,
-                        counters, emit_sums, out->capacity, tk_a, emit_vals, tile_passes, hist + 4 * 256, vn,
-                        out->status)))
+    if ((s = launch_pdl(emit_kernel, (int)std::min<int64_t>(nbe, kSMs * 8), kEmitBlock, 0, st, vt, sorted_items,
+                        proj->tiles_touched, uvdo, conic, counters, emit_sums, out->capacity, tk_a, emit_vals, tile_passes,
+                        digit_bits, hist + 4 * 256, vn, out->status)))
         return s;
     if (out->capacity == 0) return write_ranges_order(tile_counts, out, total_tiles, st);
 
     // 4. stable sort of the instances by tile id
-    if ((s = radix_sort<kSortThreadsInst, kSortIPTInst>({tk_a, emit_vals, tk_b, other_vals}, counters + CTR_M, out->capacity, tile_passes,
-                        hist + 4 * 256, lookback + (size_t)4 * L.lb_tiles_depth * 256, L.lb_tiles_inst,
-                        counters + CTR_TILE + 4, out->status, prm.spin_limit, st, tile_counts, (uint32_t)total_tiles)))
-        return s;
+    auto tile_sort = [&](auto bits) {
+        return radix_sort<kSortThreadsInst, kSortIPTInst, decltype(bits)::value>(
+            {tk_a, emit_vals, tk_b, other_vals}, counters + CTR_M, out->capacity, tile_passes, hist + 4 * 256,
+            lookback + (size_t)4 * L.lb_tiles_depth * 256, L.lb_tiles_inst, counters + CTR_TILE + 4, out->status,
+            prm.spin_limit, st, tile_counts, (uint32_t)total_tiles);
+    };
+    s = digit_bits == 5   ? tile_sort(std::integral_constant<int, 5>())
+        : digit_bits == 6 ? tile_sort(std::integral_constant<int, 6>())
+        : digit_bits == 7 ? tile_sort(std::integral_constant<int, 7>())
+                          : tile_sort(std::integral_constant<int, 8>());
+    if (s) return s;
     const uint32_t *sorted_tiles = (tile_passes % 2 == 0) ? tk_a : tk_b;
 
     // 5. per-tile ranges from the tile counts, the launch order, and the 64-bit keys if requested

@@ -27,7 +27,7 @@ struct Shape {
     bool ok;
 };
 
-__device__ __forceinline__ void load_shape(const float *quats, const float *log_scales, int64_t g, Shape &sh) {
+__device__ __forceinline__ void load_shape(const float *quats, const float *log_scales, uint32_t g, Shape &sh) {
     float4 q = reinterpret_cast<const float4 *>(quats)[g];
     sh.qn = sqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
     sh.ok = sh.qn > 0.f;
@@ -35,7 +35,7 @@ __device__ __forceinline__ void load_shape(const float *quats, const float *log_
     sh.qh[0] = q.x * inv; sh.qh[1] = q.y * inv; sh.qh[2] = q.z * inv; sh.qh[3] = q.w * inv;
     quat_rot(sh.qh, sh.Rq);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) sh.s[c] = expf(log_scales[3 * g + c]);
+    for (int c = 0; c < 3; ++c) sh.s[c] = expf(log_scales[3 * (size_t)g + c]);
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -135,7 +135,10 @@ __device__ __forceinline__ void project_geo(const float mu[3], const Shape &sh, 
     o.ok = isfinite(o.u) && isfinite(o.v) && isfinite(o.A) && isfinite(o.B) && isfinite(o.C);
 }
 
-__global__ void __launch_bounds__(256) project_fwd_kernel(ViewTable vt, Params prm, int64_t n,
+// A thread projects its Gaussian into views [blockIdx.y * per, (blockIdx.y + 1) * per): the parameters are
+// read, activated and turned into the 3D covariance once for all of them.  Bound by instruction issue
+// (84 % of cycles; the compensated centre, the activation and the covariance products).
+__global__ void __launch_bounds__(256, 6) project_fwd_kernel(ViewTable vt, Params prm, uint32_t n, int per,
                                                           const float *__restrict__ means,
                                                           const float *__restrict__ quats,
                                                           const float *__restrict__ log_scales,
@@ -145,153 +148,134 @@ __global__ void __launch_bounds__(256) project_fwd_kernel(ViewTable vt, Params p
                                                           int32_t *__restrict__ touched) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int v = blockIdx.y;
+    const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n) return;
-    int64_t item = (int64_t)v * n + g;
     Shape sh;
     load_shape(quats, log_scales, g, sh);
     float mu[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
     float o = 1.f / (1.f + expf(-logits[g]));
-    float R[9], t[3];
-    load_pose(vt, pose_dev, v, R, t);
-    Geo ge;
-    project_geo(mu, sh, R, t, vt, v, prm, ge, true);
-    float4 rec = make_float4(0.f, 0.f, ge.p[2], o);
-    float2 lo = make_float2(0.f, 0.f);
-    float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
-    int tt = 0;
-    if (ge.ok) {
-        float mid = 0.5f * (ge.a + ge.c);
-        float det = ge.a * ge.c - ge.b * ge.b;
-        float lmax = mid + sqrtf(fmaxf(mid * mid - det, 0.f));
-        float rr = fminf(prm.radius_sigma * sqrtf(lmax), 16777216.f);
-        int r = (int)ceilf(rr);
-        if (r > 0) {
-            int x0, y0, x1, y1;
-            tile_rect(ge.u, ge.v, r, vt.TX[v], vt.TY[v], x0, y0, x1, y1);
-            tt = (x1 - x0) * (y1 - y0);
+    const int v_end = min((int)(blockIdx.y + 1) * per, vt.n_views);
+#pragma unroll 1
+    for (int v = blockIdx.y * per; v < v_end; ++v) {
+        const uint32_t item = (uint32_t)v * n + g;
+        float R[9], t[3];
+        load_pose(vt, pose_dev, v, R, t);
+        Geo ge;
+        project_geo(mu, sh, R, t, vt, v, prm, ge, true);
+        float4 rec = make_float4(0.f, 0.f, ge.p[2], o);
+        float2 lo = make_float2(0.f, 0.f);
+        float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
+        int tt = 0;
+        if (ge.ok) {
+            float mid = 0.5f * (ge.a + ge.c);
+            float det = ge.a * ge.c - ge.b * ge.b;
+            float lmax = mid + sqrtf(fmaxf(mid * mid - det, 0.f));
+            float rr = fminf(prm.radius_sigma * sqrtf(lmax), 16777216.f);
+            int r = (int)ceilf(rr);
+            if (r > 0) {
+                int x0, y0, x1, y1;
+                tile_rect(ge.u, ge.v, r, vt.TX[v], vt.TY[v], x0, y0, x1, y1);
+                tt = (x1 - x0) * (y1 - y0);
+            }
+            rec.x = ge.u;
+            rec.y = ge.v;
+            lo = make_float2(ge.ulo, ge.vlo);
+            cn = make_float4(ge.A, ge.B, ge.C, (float)r);
         }
-        rec.x = ge.u;
-        rec.y = ge.v;
-        lo = make_float2(ge.ulo, ge.vlo);
-        cn = make_float4(ge.A, ge.B, ge.C, (float)r);
+        uvdo[item] = rec;
+        uv_lo[item] = lo;
+        conic[item] = cn;
+        touched[item] = tt;
     }
-    uvdo[item] = rec;
-    uv_lo[item] = lo;
-    conic[item] = cn;
-    touched[item] = tt;
 }
 
-// Register cap: six 128-thread blocks per SM (80 registers, 16 bytes spilled) instead of
-// four at 124 registers: the kernel is latency-bound and the extra warps hide it (five
-// blocks at 96 registers: -13 %; six: a further -8 %; seven spill 80 bytes).
-__global__ void __launch_bounds__(128, 6) project_bwd_kernel(ViewTable vt, Params prm, int64_t n,
-                                                          const float *__restrict__ means,
-                                                          const float *__restrict__ quats,
-                                                          const float *__restrict__ log_scales,
-                                                          const float *__restrict__ logits,
-                                                          const float *__restrict__ pose_dev,
-                                                          const float4 *__restrict__ acc_uvod,
-                                                          const float4 *__restrict__ acc_conic,
-                                                          const float4 *__restrict__ acc_rgb, int grad_mode,
-                                                          float *__restrict__ d_means, float *__restrict__ d_quats,
-                                                          float *__restrict__ d_log_scales,
-                                                          float *__restrict__ d_logits, float *__restrict__ d_rgb,
-                                                          float *__restrict__ pose_part) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n) return;
-    Shape sh;
-    load_shape(quats, log_scales, g, sh);
-    float mu[3] = {means[3 * g], means[3 * g + 1], means[3 * g + 2]};
-    float gmu[3] = {0.f, 0.f, 0.f};
-    float GS[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // dL/dSigma (trace form)
-    float dop = 0.f;
-    for (int v = 0; v < vt.n_views; ++v) {
-        int64_t item = (int64_t)v * n + g;
-        float4 a0 = acc_uvod[item], a1 = acc_conic[item];
-        float tw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        bool any = (a0.x != 0.f) | (a0.y != 0.f) | (a0.z != 0.f) | (a0.w != 0.f) | (a1.x != 0.f) | (a1.y != 0.f) |
-                   (a1.z != 0.f);
-        if (any) {
-            float R[9], t[3];
-            load_pose(vt, pose_dev, v, R, t);
-            float fx = vt.fx[v], fy = vt.fy[v];
-            Geo ge;
-            project_geo(mu, sh, R, t, vt, v, prm, ge);
-            if (ge.ok) {
-                dop += a0.z;
-                // conic -> Sigma2D: G2 = -conic Ghat conic, Ghat = [[dA, dB/2], [dB/2, dC]]
-                float hA = a1.x, hB = 0.5f * a1.y, hC = a1.z;
-                float X00 = ge.A * hA + ge.B * hB, X01 = ge.A * hB + ge.B * hC;
-                float X10 = ge.B * hA + ge.C * hB, X11 = ge.B * hB + ge.C * hC;
-                float g00 = -(X00 * ge.A + X01 * ge.B);
-                float g01 = -(X00 * ge.B + X01 * ge.C);
-                float g11 = -(X10 * ge.B + X11 * ge.C);
-                // Sigma2D = J Sc J^T: Gc = J^T G2 J, dJ = 2 G2 J Sc
-                Cov3 Gc;
-                Gc.m[0] = ge.j00 * ge.j00 * g00;
-                Gc.m[1] = ge.j00 * ge.j11 * g01;
-                Gc.m[2] = ge.j00 * (ge.j02 * g00 + ge.j12 * g01);
-                Gc.m[3] = ge.j11 * ge.j11 * g11;
-                Gc.m[4] = ge.j11 * (ge.j02 * g01 + ge.j12 * g11);
-                Gc.m[5] = ge.j02 * ge.j02 * g00 + 2.f * ge.j02 * ge.j12 * g01 + ge.j12 * ge.j12 * g11;
-                const float *S = ge.Sc.m;
-                float JS0[3] = {ge.j00 * S[0] + ge.j02 * S[2], ge.j00 * S[1] + ge.j02 * S[4], ge.j00 * S[2] + ge.j02 * S[5]};
-                float JS1[3] = {ge.j11 * S[1] + ge.j12 * S[2], ge.j11 * S[3] + ge.j12 * S[4], ge.j11 * S[4] + ge.j12 * S[5]};
-                float dJ00 = 2.f * (g00 * JS0[0] + g01 * JS1[0]);
-                float dJ02 = 2.f * (g00 * JS0[2] + g01 * JS1[2]);
-                float dJ11 = 2.f * (g01 * JS0[1] + g11 * JS1[1]);
-                float dJ12 = 2.f * (g01 * JS0[2] + g11 * JS1[2]);
-                // camera-frame centre
-                float x = ge.p[0], y = ge.p[1], z = ge.p[2];
-                float iz = 1.f / z, iz2 = iz * iz;
-                // J02 = -fx t_x / z with t_x = clamp(x / z): dt_x/dx = 1/z, dt_x/dz = -x/z^2 inside, 0 outside
-                const float dtx_dx = ge.in_x ? iz : 0.f, dtx_dz = ge.in_x ? -x * iz2 : 0.f;
-                const float dty_dy = ge.in_y ? iz : 0.f, dty_dz = ge.in_y ? -y * iz2 : 0.f;
-                float gp0 = a0.x * fx * iz + dJ02 * (-fx * iz) * dtx_dx;
-                float gp1 = a0.y * fy * iz + dJ12 * (-fy * iz) * dty_dy;
-                float gp2 = -a0.x * fx * x * iz2 - a0.y * fy * y * iz2 + a0.w + dJ00 * (-fx * iz2) +
-                            dJ02 * (-fx * dtx_dz * iz + fx * ge.tx * iz2) + dJ11 * (-fy * iz2) +
-                            dJ12 * (-fy * dty_dz * iz + fy * ge.ty * iz2);
+// Gradients of one Gaussian collected over the views: its mean, Sigma (trace form) and activated opacity.
+struct GaussSums {
+    float gmu[3], GS[9], dop;
+};
+
+// Adds one view's splat sums (a0: centre, opacity, depth; a1: conic) of Gaussian (mu, sh), and with `pose` forms
+// the view's twist parts.
+__device__ __forceinline__ void project_view_bwd(const ViewTable &vt, const Params &prm, const float *pose_dev, int v,
+                                                 const float mu[3], const Shape &sh, float4 a0, float4 a1, bool pose,
+                                                 GaussSums &out, float tw[6]) {
+    float R[9], t[3];
+    load_pose(vt, pose_dev, v, R, t);
+    const float fx = vt.fx[v], fy = vt.fy[v];
+    Geo ge;
+    project_geo(mu, sh, R, t, vt, v, prm, ge);
+    if (!ge.ok) return;
+    out.dop += a0.z;
+    // conic -> Sigma2D: G2 = -conic Ghat conic, Ghat = [[dA, dB/2], [dB/2, dC]]
+    float hA = a1.x, hB = 0.5f * a1.y, hC = a1.z;
+    float X00 = ge.A * hA + ge.B * hB, X01 = ge.A * hB + ge.B * hC;
+    float X10 = ge.B * hA + ge.C * hB, X11 = ge.B * hB + ge.C * hC;
+    float g00 = -(X00 * ge.A + X01 * ge.B);
+    float g01 = -(X00 * ge.B + X01 * ge.C);
+    float g11 = -(X10 * ge.B + X11 * ge.C);
+    // Sigma2D = J Sc J^T: Gc = J^T G2 J, dJ = 2 G2 J Sc
+    Cov3 Gc;
+    Gc.m[0] = ge.j00 * ge.j00 * g00;
+    Gc.m[1] = ge.j00 * ge.j11 * g01;
+    Gc.m[2] = ge.j00 * (ge.j02 * g00 + ge.j12 * g01);
+    Gc.m[3] = ge.j11 * ge.j11 * g11;
+    Gc.m[4] = ge.j11 * (ge.j02 * g01 + ge.j12 * g11);
+    Gc.m[5] = ge.j02 * ge.j02 * g00 + 2.f * ge.j02 * ge.j12 * g01 + ge.j12 * ge.j12 * g11;
+    const float *S = ge.Sc.m;
+    float JS0[3] = {ge.j00 * S[0] + ge.j02 * S[2], ge.j00 * S[1] + ge.j02 * S[4], ge.j00 * S[2] + ge.j02 * S[5]};
+    float JS1[3] = {ge.j11 * S[1] + ge.j12 * S[2], ge.j11 * S[3] + ge.j12 * S[4], ge.j11 * S[4] + ge.j12 * S[5]};
+    float dJ00 = 2.f * (g00 * JS0[0] + g01 * JS1[0]);
+    float dJ02 = 2.f * (g00 * JS0[2] + g01 * JS1[2]);
+    float dJ11 = 2.f * (g01 * JS0[1] + g11 * JS1[1]);
+    float dJ12 = 2.f * (g01 * JS0[2] + g11 * JS1[2]);
+    // camera-frame centre
+    float x = ge.p[0], y = ge.p[1], z = ge.p[2];
+    float iz = 1.f / z, iz2 = iz * iz;
+    // J02 = -fx t_x / z with t_x = clamp(x / z): dt_x/dx = 1/z, dt_x/dz = -x/z^2 inside, 0 outside
+    const float dtx_dx = ge.in_x ? iz : 0.f, dtx_dz = ge.in_x ? -x * iz2 : 0.f;
+    const float dty_dy = ge.in_y ? iz : 0.f, dty_dz = ge.in_y ? -y * iz2 : 0.f;
+    float gp0 = a0.x * fx * iz + dJ02 * (-fx * iz) * dtx_dx;
+    float gp1 = a0.y * fy * iz + dJ12 * (-fy * iz) * dty_dy;
+    float gp2 = -a0.x * fx * x * iz2 - a0.y * fy * y * iz2 + a0.w + dJ00 * (-fx * iz2) +
+                dJ02 * (-fx * dtx_dz * iz + fx * ge.tx * iz2) + dJ11 * (-fy * iz2) +
+                dJ12 * (-fy * dty_dz * iz + fy * ge.ty * iz2);
 #pragma unroll
-                for (int k = 0; k < 3; ++k) gmu[k] += R[k] * gp0 + R[3 + k] * gp1 + R[6 + k] * gp2;
-                // Sigma gradient: R^T Gc R
-                float GR[9];
+    for (int k = 0; k < 3; ++k) out.gmu[k] += R[k] * gp0 + R[3 + k] * gp1 + R[6 + k] * gp2;
+    // Sigma gradient: R^T Gc R
+    float GR[9];
 #pragma unroll
-                for (int r = 0; r < 3; ++r)
+    for (int r = 0; r < 3; ++r)
 #pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        GR[3 * r + k] = sym(Gc, r, 0) * R[k] + sym(Gc, r, 1) * R[3 + k] + sym(Gc, r, 2) * R[6 + k];
+        for (int k = 0; k < 3; ++k)
+            GR[3 * r + k] = sym(Gc, r, 0) * R[k] + sym(Gc, r, 1) * R[3 + k] + sym(Gc, r, 2) * R[6 + k];
+    const int sr[6] = {0, 0, 0, 1, 1, 2}, sk[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
-                for (int r = 0; r < 3; ++r)
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) GS[3 * r + k] += R[r] * GR[k] + R[3 + r] * GR[3 + k] + R[6 + r] * GR[6 + k];
-                if (grad_mode & GS_GRAD_POSE) {
-                    // A = Sc Gc - Gc Sc (antisymmetric); twist phi gets p x g_p + 2 (A12, A20, A01)
-                    auto prod = [&](int r, int k) {
-                        return sym(ge.Sc, r, 0) * sym(Gc, 0, k) + sym(ge.Sc, r, 1) * sym(Gc, 1, k) +
-                               sym(ge.Sc, r, 2) * sym(Gc, 2, k);
-                    };
-                    float A12 = prod(1, 2) - prod(2, 1);
-                    float A20 = prod(2, 0) - prod(0, 2);
-                    float A01 = prod(0, 1) - prod(1, 0);
-                    tw[0] = gp0; tw[1] = gp1; tw[2] = gp2;
-                    tw[3] = y * gp2 - z * gp1 + 2.f * A12;
-                    tw[4] = z * gp0 - x * gp2 + 2.f * A20;
-                    tw[5] = x * gp1 - y * gp0 + 2.f * A01;
-                }
-            }
-        }
-        if (grad_mode & GS_GRAD_POSE) {
-#pragma unroll
-            for (int k = 0; k < 6; ++k) pose_part[((int64_t)v * 6 + k) * n + g] = tw[k];
-        }
+    for (int e = 0; e < 6; ++e)
+        out.GS[e] += R[sr[e]] * GR[sk[e]] + R[3 + sr[e]] * GR[3 + sk[e]] + R[6 + sr[e]] * GR[6 + sk[e]];
+    if (pose) {
+        // A = Sc Gc - Gc Sc (antisymmetric); twist phi gets p x g_p + 2 (A12, A20, A01)
+        auto prod = [&](int r, int k) {
+            return sym(ge.Sc, r, 0) * sym(Gc, 0, k) + sym(ge.Sc, r, 1) * sym(Gc, 1, k) +
+                   sym(ge.Sc, r, 2) * sym(Gc, 2, k);
+        };
+        float A12 = prod(1, 2) - prod(2, 1);
+        float A20 = prod(2, 0) - prod(0, 2);
+        float A01 = prod(0, 1) - prod(1, 0);
+        tw[0] = gp0; tw[1] = gp1; tw[2] = gp2;
+        tw[3] = y * gp2 - z * gp1 + 2.f * A12;
+        tw[4] = z * gp0 - x * gp2 + 2.f * A20;
+        tw[5] = x * gp1 - y * gp0 + 2.f * A01;
     }
-    if (!(grad_mode & GS_GRAD_MAP)) return;
-    // Sigma = M M^T -> M -> (s, Rq) -> q
+}
+
+struct BwdOut {
+    float *means, *quats, *log_scales, *logits, *rgb, *pose_part;
+};
+
+// From the collected sums to the parameters: Sigma = M M^T -> M -> (s, Rq) -> q, and the rest.
+__device__ __forceinline__ void write_gauss_grads(const Shape &sh, const GaussSums &a, float logit, uint32_t g,
+                                                  const BwdOut &o) {
+    const float GS[9] = {a.GS[0], a.GS[1], a.GS[2], a.GS[1], a.GS[3], a.GS[4], a.GS[2], a.GS[4], a.GS[5]};
     float dM[9];
 #pragma unroll
     for (int r = 0; r < 3; ++r)
@@ -302,7 +286,7 @@ __global__ void __launch_bounds__(128, 6) project_bwd_kernel(ViewTable vt, Param
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         float ds = dM[k] * sh.Rq[k] + dM[3 + k] * sh.Rq[3 + k] + dM[6 + k] * sh.Rq[6 + k];
-        d_log_scales[3 * g + k] = ds * sh.s[k];
+        o.log_scales[3 * (size_t)g + k] = ds * sh.s[k];
 #pragma unroll
         for (int r = 0; r < 3; ++r) dR[3 * r + k] = dM[3 * r + k] * sh.s[k];
     }
@@ -316,15 +300,122 @@ __global__ void __launch_bounds__(128, 6) project_bwd_kernel(ViewTable vt, Param
     float iq = sh.ok ? 1.f / sh.qn : 0.f;
     float4 dq = make_float4((gq[0] - sh.qh[0] * dot) * iq, (gq[1] - sh.qh[1] * dot) * iq,
                             (gq[2] - sh.qh[2] * dot) * iq, (gq[3] - sh.qh[3] * dot) * iq);
-    reinterpret_cast<float4 *>(d_quats)[g] = dq;
+    reinterpret_cast<float4 *>(o.quats)[g] = dq;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) d_means[3 * g + k] = gmu[k];
-    float o = 1.f / (1.f + expf(-logits[g]));
-    d_logits[g] = o * (1.f - o) * dop;
-    float4 cr = acc_rgb[g];
-    d_rgb[3 * g] = cr.x;
-    d_rgb[3 * g + 1] = cr.y;
-    d_rgb[3 * g + 2] = cr.z;
+    for (int k = 0; k < 3; ++k) o.means[3 * (size_t)g + k] = a.gmu[k];
+    const float op = 1.f / (1.f + expf(-logit));
+    o.logits[g] = op * (1.f - op) * a.dop;
+}
+
+// One view: the Gaussians are walked by warps, SPAN at a time.  Most of a map is out of a frame (82 % of the room at
+// 1200x680) and has zero sums, spread over the index space: with a Gaussian per lane nearly every warp ran the
+// whole chain for a fifth of its lanes.  A warp instead reads the splat sums of its span (coalesced),
+// writes the zeros, lists the Gaussians that have a gradient, and runs the chain on 32 listed ones at a time.
+constexpr int kBwdWarps = 4;
+
+template <int SPAN>
+__global__ void __launch_bounds__(32 * kBwdWarps, 6) project_bwd_one_kernel(
+    ViewTable vt, Params prm, uint32_t n, const float *__restrict__ means, const float *__restrict__ quats,
+    const float *__restrict__ log_scales, const float *__restrict__ logits, const float *__restrict__ pose_dev,
+    const float4 *__restrict__ acc_uvod, const float4 *__restrict__ acc_conic, const float4 *__restrict__ acc_rgb,
+    int grad_mode, BwdOut out) {
+    pdl_wait();     // the previous kernel's results
+    pdl_trigger();  // the next kernel may be scheduled now
+    constexpr int ROUNDS = SPAN / 32;
+    static_assert(SPAN % 32 == 0 && SPAN <= 256, "list entries are bytes");
+    __shared__ uint8_t s_list[kBwdWarps][SPAN];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint64_t first = ((uint64_t)blockIdx.x * kBwdWarps + w) * SPAN;
+    if (first >= n) return;  // whole warp; no block barrier below
+    const uint32_t g0 = (uint32_t)first + lane;  // this lane's Gaussians: g0 + 32 r
+    const bool map = grad_mode & GS_GRAD_MAP, pose = grad_mode & GS_GRAD_POSE;
+    uint8_t *list = s_list[w];
+    int cnt = 0;
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const uint32_t g = g0 + 32 * r;
+        bool any = false;
+        if (g < n) {
+            const float4 a0 = acc_uvod[g], a1 = acc_conic[g];
+            any = (a0.x != 0.f) | (a0.y != 0.f) | (a0.z != 0.f) | (a0.w != 0.f) | (a1.x != 0.f) | (a1.y != 0.f) |
+                  (a1.z != 0.f);
+            if (map) {
+                const float4 cr = acc_rgb[g];
+                out.rgb[3 * (size_t)g] = cr.x;
+                out.rgb[3 * (size_t)g + 1] = cr.y;
+                out.rgb[3 * (size_t)g + 2] = cr.z;
+                if (!any) {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) out.means[3 * (size_t)g + k] = out.log_scales[3 * (size_t)g + k] = 0.f;
+                    reinterpret_cast<float4 *>(out.quats)[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    out.logits[g] = 0.f;
+                }
+            }
+            if (pose && !any) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k) out.pose_part[(size_t)k * n + g] = 0.f;
+            }
+        }
+        const uint32_t bal = __ballot_sync(0xffffffffu, any);
+        if (any) list[cnt + __popc(bal & lanemask_lt())] = (uint8_t)(32 * r + lane);
+        cnt += __popc(bal);
+    }
+    __syncwarp();
+    for (int at = lane; at < cnt; at += 32) {
+        const uint32_t g = (uint32_t)first + list[at];
+        Shape sh;
+        load_shape(quats, log_scales, g, sh);
+        const float mu[3] = {means[3 * (size_t)g], means[3 * (size_t)g + 1], means[3 * (size_t)g + 2]};
+        GaussSums a = {};
+        float tw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        project_view_bwd(vt, prm, pose_dev, 0, mu, sh, acc_uvod[g], acc_conic[g], pose, a, tw);
+        if (pose) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) out.pose_part[(size_t)k * n + g] = tw[k];
+        }
+        if (map) write_gauss_grads(sh, a, logits[g], g, out);
+    }
+}
+
+// Several views: one thread per Gaussian, looping over the views (lists per view with the sums in shared memory
+// took 0.367 against 0.327 ms for 2M Gaussians in eight views: every listed pair activates its Gaussian anew).
+// Register cap: six 128-thread blocks per SM (80 registers) instead of four at 124: the kernel is
+// latency-bound and the extra warps hide it (five blocks at 96 registers: -13 %; six: a further -8 %).
+__global__ void __launch_bounds__(128, 6) project_bwd_kernel(ViewTable vt, Params prm, uint32_t n,
+                                                             const float *__restrict__ means,
+                                                             const float *__restrict__ quats,
+                                                             const float *__restrict__ log_scales,
+                                                             const float *__restrict__ logits,
+                                                             const float *__restrict__ pose_dev,
+                                                             const float4 *__restrict__ acc_uvod,
+                                                             const float4 *__restrict__ acc_conic,
+                                                             const float4 *__restrict__ acc_rgb, int grad_mode, BwdOut out) {
+    pdl_wait();     // the previous kernel's results
+    pdl_trigger();  // the next kernel may be scheduled now
+    const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n) return;
+    const bool map = grad_mode & GS_GRAD_MAP, pose = grad_mode & GS_GRAD_POSE;
+    Shape sh;
+    load_shape(quats, log_scales, g, sh);
+    const float mu[3] = {means[3 * (size_t)g], means[3 * (size_t)g + 1], means[3 * (size_t)g + 2]};
+    GaussSums a = {};
+    for (int v = 0; v < vt.n_views; ++v) {
+        const size_t item = (size_t)v * n + g;
+        const float4 a0 = acc_uvod[item], a1 = acc_conic[item];
+        float tw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if ((a0.x != 0.f) | (a0.y != 0.f) | (a0.z != 0.f) | (a0.w != 0.f) | (a1.x != 0.f) | (a1.y != 0.f) | (a1.z != 0.f))
+            project_view_bwd(vt, prm, pose_dev, v, mu, sh, a0, a1, pose, a, tw);
+        if (pose) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) out.pose_part[((size_t)v * 6 + k) * n + g] = tw[k];
+        }
+    }
+    if (!map) return;
+    write_gauss_grads(sh, a, logits[g], g, out);
+    const float4 cr = acc_rgb[g];
+    out.rgb[3 * (size_t)g] = cr.x;
+    out.rgb[3 * (size_t)g + 1] = cr.y;
+    out.rgb[3 * (size_t)g + 2] = cr.z;
 }
 
 }  // namespace
@@ -348,8 +439,14 @@ extern "C" gs_status gs_project(const gs_gaussians *g, const gs_camera *cams, in
     if ((reinterpret_cast<uintptr_t>(g->quats) | reinterpret_cast<uintptr_t>(out->uvdo) |
          reinterpret_cast<uintptr_t>(out->conic)) & 15 || (reinterpret_cast<uintptr_t>(out->uv_lo) & 7))
         return GS_ERR_ARG;
-    dim3 grid(ceil_div(g->n, 256), n_views);
-    return launch_pdl(project_fwd_kernel, grid, 256, 0, (cudaStream_t)stream, vt, prm, g->n, g->means, g->quats,
+    // views per thread: all of them once the Gaussians alone fill the GPU twice over, fewer for a small field.
+    // One view per thread took 0.128 ms for 1M Gaussians in six views and 0.344 for 2M in eight; sharing the
+    // parameters and the covariance over the views takes 0.093 and 0.235.
+    const int64_t threads = 2 * (int64_t)kSMs * 2048;
+    const int groups = (int)std::min<int64_t>(n_views, (threads + g->n - 1) / g->n);
+    const int per = (n_views + groups - 1) / groups;
+    dim3 grid(ceil_div(g->n, 256), (n_views + per - 1) / per);
+    return launch_pdl(project_fwd_kernel, grid, 256, 0, (cudaStream_t)stream, vt, prm, (uint32_t)g->n, per, g->means, g->quats,
                       g->log_scales, g->opacity_logits, pose_dev, reinterpret_cast<float4 *>(out->uvdo),
                       reinterpret_cast<float2 *>(out->uv_lo), reinterpret_cast<float4 *>(out->conic),
                       out->tiles_touched);
@@ -378,11 +475,19 @@ extern "C" gs_status gs_project_bwd(const gs_gaussians *g, const gs_camera *cams
          reinterpret_cast<uintptr_t>(sg->conic) | reinterpret_cast<uintptr_t>(sg->rgb) |
          reinterpret_cast<uintptr_t>(map ? out->quats : nullptr)) & 15)
         return GS_ERR_ARG;
-    dim3 grid(ceil_div(g->n, 128));
-    return launch_pdl(project_bwd_kernel, grid, 128, 0, (cudaStream_t)stream, vt, prm, g->n, g->means, g->quats,
-                      g->log_scales, g->opacity_logits, pose_dev, reinterpret_cast<const float4 *>(sg->uvod),
-                      reinterpret_cast<const float4 *>(sg->conic), reinterpret_cast<const float4 *>(sg->rgb),
-                      grad_mode, map ? out->means : nullptr, map ? out->quats : nullptr,
-                      map ? out->log_scales : nullptr, map ? out->opacity_logits : nullptr,
-                      map ? out->rgb : nullptr, pose ? pose_part : nullptr);
+    const BwdOut o{map ? out->means : nullptr,          map ? out->quats : nullptr, map ? out->log_scales : nullptr,
+                   map ? out->opacity_logits : nullptr, map ? out->rgb : nullptr,   pose ? pose_part : nullptr};
+    auto launch = [&](auto kern, int per_block) {
+        return launch_pdl(kern, ceil_div(g->n, per_block), 128, 0, (cudaStream_t)stream, vt, prm, (uint32_t)g->n, g->means,
+                          g->quats, g->log_scales, g->opacity_logits, pose_dev, reinterpret_cast<const float4 *>(sg->uvod),
+                          reinterpret_cast<const float4 *>(sg->conic), reinterpret_cast<const float4 *>(sg->rgb), grad_mode,
+                          o);
+    };
+    if (n_views > 1) return launch(project_bwd_kernel, 128);
+    // spans as long as the resident warps (24 per SM) are filled: 1M Gaussians at 1200x680 0.034 ms with 128 (0.036,
+    // 0.037, 0.046 with 256, 64, 32; 0.048 with a Gaussian per lane), at 640x480 0.027 (0.045)
+    const int64_t fill = g->n / (24 * kSMs);
+    return fill >= 128  ? launch(project_bwd_one_kernel<128>, 128 * kBwdWarps)
+           : fill >= 64 ? launch(project_bwd_one_kernel<64>, 64 * kBwdWarps)
+                        : launch(project_bwd_one_kernel<32>, 32 * kBwdWarps);
 }

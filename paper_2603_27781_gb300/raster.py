@@ -81,8 +81,19 @@ def _p(t: Optional[torch.Tensor]):
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    # the raw handle (0.7 us) rather than a Stream object around it (3 us): once per call into libgs
+    if stream is None:
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return ctypes.c_void_p(stream.cuda_stream)
+
+
+def _copies(tensors):
+    """Contiguous copies of a list of tensors by one launch where they are dense and of one type (a
+    clone each costs 7 us of host time and a copy of its own on the device)."""
+    out = [torch.empty(t.shape, dtype=t.dtype, device=t.device) for t in tensors]
+    with torch.no_grad():
+        torch._foreach_copy_(out, tensors)
+    return out
 
 
 _DTYPE = {torch.float32: L.GS_F32, torch.float16: L.GS_F16, torch.bfloat16: L.GS_BF16}
@@ -534,25 +545,31 @@ def expand(r: "Renderer", field: Field, targets, feat_init: torch.Tensor, tau_un
         raise ValueError("expansion appends to f32 parameter storage")
     n, D = field.n, field.feat_dim
     n_max = int(feat_init.shape[0])
-    grow = lambda t: torch.cat([t, t.new_zeros((n_max,) + tuple(t.shape[1:]))]).contiguous()
-    out = Field(*(grow(t) for t in (field.means, field.quats, field.log_scales, field.opacity_logits, field.rgb,
-                                    field.feat)))
+    # rows [0, n) are copied by one launch, the rows after them are written by the kernel (six
+    # concatenations with zeros, 27 us of host time each, were most of the call's 400 us)
+    old = [field.means, field.quats, field.log_scales, field.opacity_logits, field.rgb, field.feat]
+    new = [t.new_empty((n + n_max,) + tuple(t.shape[1:])) for t in old]
+    if torch.is_grad_enabled() and any(t.requires_grad for t in old):
+        for t, o in zip(new, old):      # the joint copy has no derivative
+            t[:n].copy_(o)
+    else:
+        torch._foreach_copy_([t[:n] for t in new], old)
+    out = Field(*new)
     fm = L.gs_field_mut(n + n_max, D, _p(out.means), _p(out.quats), _p(out.log_scales), _p(out.opacity_logits),
                         _p(out.rgb), _p(out.feat) if D else None)
     dev = field.means.device
-    n_new = torch.zeros(1, dtype=torch.int64, device=dev)
-    src = torch.zeros(max(n_max, 1), dtype=torch.int64, device=dev)
-    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    # the count [8 bytes] and the status word [4 bytes], both written by the call, read back together
+    result = torch.empty(3, dtype=torch.int32, device=dev)
+    src = torch.empty(max(n_max, 1), dtype=torch.int64, device=dev)
     tc = L.gs_targets(_p(targets["rgb"]), _p(targets["depth"]), _p(targets["label"]))
     fi = feat_init.contiguous().to(torch.float32)
     L.check("gs_expand", L.gs_expand(r.cams_c, r.n_views, ctypes.byref(r.images_c()), ctypes.byref(tc), tau_unobs,
-                                     _p(fi) if D else None, n, ctypes.byref(fm), _p(n_new), _p(src), _p(status),
-                                     _p(r.ws), r.ws.numel(), _stream(stream)))
-    total = int(n_new.item())
+                                     _p(fi) if D else None, n, ctypes.byref(fm), _p(result), _p(src),
+                                     _p(result[2:]), _p(r.ws), r.ws.numel(), _stream(stream)))
+    lo, hi, status = result.tolist()
+    total = hi << 32 | (lo & 0xffffffff)
     k = min(total, n_max)
-    keep = lambda t: t[: n + k].contiguous()
-    return Field(*(keep(t) for t in (out.means, out.quats, out.log_scales, out.opacity_logits, out.rgb,
-                                     out.feat))), src[:k], total, int(status.item())
+    return Field(*(t[: n + k] for t in new)), src[:k], total, status
 
 
 class Tracker:
@@ -652,22 +669,23 @@ class RasterizeSG(torch.autograd.Function):
         renderer.forward(field)
         ctx.renderer, ctx.field = renderer, field
         D = renderer.feat_dim
-        return (renderer.img_rgb.clone(), renderer.img_depth.clone(), renderer.img_sil.clone(),
-                renderer.img_feat[:D].clone())
+        return tuple(_copies([renderer.img_rgb, renderer.img_depth, renderer.img_sil, renderer.img_feat[:D]]))
 
     @staticmethod
     def backward(ctx, g_rgb, g_depth, g_sil, g_feat):
         r = ctx.renderer
-        z = lambda g, like: like.zero_() if g is None else like.copy_(g)
-        z(g_rgb, r.g_rgb)
-        z(g_depth, r.g_depth)
-        z(g_sil, r.g_sil)
-        if r.feat_dim:
-            z(g_feat, r.g_feat[: r.feat_dim])
-        r.backward(ctx.field, L.GS_GRAD_MAP)
         D = r.feat_dim
-        return (None, r.d_means.clone(), r.d_quats.clone(), r.d_log_scales.clone(), r.d_logits.clone(),
-                r.d_rgb.clone(), r.d_feat[:, :D].clone() if D else torch.zeros_like(ctx.field.feat))
+        bufs = [(r.g_rgb, g_rgb), (r.g_depth, g_depth), (r.g_sil, g_sil)] + ([(r.g_feat[:D], g_feat)] if D else [])
+        given = [(b, g) for b, g in bufs if g is not None]
+        if given:
+            with torch.no_grad():       # also under create_graph: nothing here has a second derivative
+                torch._foreach_copy_([b for b, _ in given], [g for _, g in given])
+        for b, g in bufs:
+            if g is None:
+                b.zero_()
+        r.backward(ctx.field, L.GS_GRAD_MAP)
+        grads = [r.d_means, r.d_quats, r.d_log_scales, r.d_logits, r.d_rgb] + ([r.d_feat[:, :D]] if D else [])
+        return (None, *_copies(grads), *(() if D else (torch.zeros_like(ctx.field.feat),)))
 
 
 def rasterize(renderer: Renderer, means, quats, log_scales, opacity_logits, rgb, feat):

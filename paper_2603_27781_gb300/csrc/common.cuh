@@ -260,6 +260,14 @@ __device__ __forceinline__ void tile_rect(float u, float v, int r, int TX, int T
 // that kernel has completed and its writes are visible, so every read of its results comes
 // after it.  pdl_trigger() lets the next kernel be launched once every block of this one has
 // called it (or exited).  Both are no-ops for a kernel launched without the attribute.
+//
+// A kernel with little to do triggers at its start: the next one's launch then hides behind it (the
+// radix passes without it: 911 against 930 us a step of 1M Gaussians at 1200x680).  The kernels that fill
+// the GPU for long do not: blocks of the next kernel that are resident and wait while the loss, the
+// blends or the instance emission run cost more than their launch.  Measured without those four
+// triggers, with them before: step at D = 32, 640x480: 581, 607 us (the loss step alone 30, 48); 1M
+// Gaussians at 1200x680: 907, 911; eight keyframes in 16-bit storage: 8.65, 8.67 ms; loss with 20
+// classes: 96, 100; view of 811x607 at D = 8: 168, 172.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

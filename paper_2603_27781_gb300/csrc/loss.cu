@@ -243,8 +243,7 @@ __global__ void __launch_bounds__(LossShape<D, KC>::NT, LossShape<D, KC>::BLOCKS
     float *__restrict__ g_depth, float *__restrict__ g_sil, float *__restrict__ g_feat, float *__restrict__ g_coef,
     float *__restrict__ part_f, double *__restrict__ part_d, float *__restrict__ mask_out,
     float *__restrict__ median_out) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
+    pdl_wait();  // the previous kernel's results (no trigger: see pdl_trigger)
     using SH = LossShape<D, KC>;
     constexpr int NT = SH::NT, NPX = SH::NPX, DD = SH::DD, TILES = SH::TILES, GROUPS = SH::GROUPS;
     __shared__ __align__(16) float s_W[KC * DD];

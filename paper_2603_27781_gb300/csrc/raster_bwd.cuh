@@ -125,8 +125,7 @@ struct BwdArgs {
 
 template <int D, int NP, bool MAP, typename RT, typename FT>
 __global__ void __launch_bounds__(Shape<NP>::THREADS) raster_bwd_kernel(ViewTable vt, Params prm, BwdArgs A) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
+    pdl_wait();  // the previous kernel's results (no trigger: see pdl_trigger)
     using LY = BwdLayout<D, NP, MAP>;
     using SH = Shape<NP>;
     constexpr int NT = SH::THREADS;

@@ -100,8 +100,7 @@ template <int D, int NP, bool MAP, int KF> constexpr int warp_bwd_min_blocks() {
 template <int D, int NP, bool MAP, int KF, typename RT, typename FT>
 __global__ void __launch_bounds__(32, warp_bwd_min_blocks<D, NP, MAP, KF>())
     raster_bwd_warp_kernel(ViewTable vt, Params prm, BwdArgs A) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
+    pdl_wait();  // the previous kernel's results (no trigger: see pdl_trigger)
     using SH = Shape<NP>;
     constexpr int STAGE = kSlots;
     using WL = WarpLayout<D, NP, MAP, KF, STAGE>;

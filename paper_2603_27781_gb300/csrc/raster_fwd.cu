@@ -284,8 +284,7 @@ __global__ void __launch_bounds__(Shape<NP>::THREADS, fwd_min_blocks(D, NP)) ras
     const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges, int64_t P, float *o_rgb, float *o_depth,
     float *o_sil, float *o_feat, float *o_T, int32_t *o_nc, int32_t *o_nb, uint32_t *bmask, int64_t bm_stride,
     const uint32_t *__restrict__ order, int32_t *status, int64_t capacity, uint32_t *queue) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
+    pdl_wait();  // the previous kernel's results (no trigger: see pdl_trigger)
     const int n_tiles = vt.tile_off[vt.n_views];
     const bool failed = binning_failed(status);  // the binning overflowed or gave up: render nothing
     if constexpr (QUEUE) {
@@ -331,8 +330,7 @@ __global__ void __launch_bounds__(32, fwd_group_min_blocks(D, NP)) raster_fwd_gr
     const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges, int64_t P, float *o_rgb, float *o_depth,
     float *o_sil, float *o_feat, float *o_T, int32_t *o_nc, int32_t *o_nb, uint32_t *bmask, int64_t bm_stride,
     const uint32_t *__restrict__ order, int32_t *status, int64_t capacity, uint32_t * /*queue*/) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
+    pdl_wait();  // the previous kernel's results (no trigger: see pdl_trigger)
     using SH = Shape<NP, true>;  // horizontal pixel pairs
     constexpr int D4 = D / 4;
     constexpr int NL = SH::PIX_GROUPS ? NP : 1;  // mask bit registers per thread
@@ -423,8 +421,7 @@ __global__ void __launch_bounds__(Shape<2, true>::THREADS, fwd_min_blocks(D, 2))
     const uint32_t *__restrict__ vals, const uint32_t *__restrict__ ranges, int64_t P, float *o_rgb, float *o_depth,
     float *o_sil, float *o_feat, float *o_T, int32_t *o_nc, int32_t *o_nb, uint32_t *bmask, int64_t bm_stride,
     const uint32_t *__restrict__ order, int32_t *status, int64_t capacity, uint32_t * /*queue*/) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
+    pdl_wait();  // the previous kernel's results (no trigger: see pdl_trigger)
     constexpr int NP = 2;
     using SH = Shape<NP, true>;  // horizontal pixel pairs
     constexpr int NT = SH::THREADS, NW = SH::WARPS;

@@ -258,8 +258,7 @@ __global__ void __launch_bounds__(kEmitBlock) emit_kernel(ViewTable vt, const ui
                                                           const uint32_t *block_sums, int64_t capacity,
                                                           uint32_t *tile_keys, uint32_t *inst_vals, int n_passes,
                                                           int bits, uint32_t *hist, int64_t vn, const int32_t *status) {
-    pdl_wait();     // the previous kernel's results
-    pdl_trigger();  // the next kernel may be scheduled now
+    pdl_wait();  // the previous kernel's results (no trigger: see pdl_trigger)
     __shared__ uint32_t s_warp[9];
     __shared__ uint32_t sh[4][256];
     __shared__ uint32_t s_off[kEmitBlock];  // exclusive instance offset of each item in the block

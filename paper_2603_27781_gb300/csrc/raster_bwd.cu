@@ -109,15 +109,16 @@ extern "C" gs_status gs_render_bwd(const gs_gaussians *g, const gs_projected *pr
     if (factored && !pr.bwd_warp) return GS_ERR_UNSUPPORTED;  // the tile kernel takes the features' gradient
     // Default pixels per thread of the per-group form: two (8x8 blocks, four per tile, whose lanes share each
     // splat's loads and shuffles over two pixels), and one (twice as many warps) where the image has too
-    // few blocks to hide latency with: below 7 two-pixel blocks per SM in map mode with the factored form,
-    // 32 (D = 16) or 20 (D = 32) otherwise, where the two-pixel kernels hold fewer warps.  Measured in ms,
-    // one against two pixels per thread:
-    //   map, factored: 0.068 / 0.096 at 64x48, 0.022 / 0.028 at 160x120, 0.070 / 0.066 at 320x240,
-    //     0.528 / 0.392 at 1200x680; D = 32: 0.279 / 0.207 at 640x480
+    // few blocks to hide latency with.  The line is in two-pixel blocks per SM, at D = 16 and 32: 24 and 16 in
+    // map mode with the factored form, 32 and 24 with the features themselves, 32 and 20 in pose mode.
+    // Measured in ms, one against two pixels per thread:
+    //   map, factored: 0.061 / 0.096 at 64x48, 0.054 / 0.065 at 320x240, 0.124 / 0.141 at 480x400, 0.096 / 0.098
+    //     at 600x384, 0.120 / 0.108 at 640x480; D = 32: 0.100 / 0.117 at 400x300, 0.111 / 0.120 and (scan) 0.244 /
+    //     0.238 at 480x400, 0.151 / 0.124 at 640x480
     //   map, features: 0.060 / 0.070 at 640x480, 0.180 / 0.164 at 811x607, 0.533 / 0.466 at 1200x680;
-    //     D = 32: 0.121 / 0.129 at 480x360, 0.373 / 0.309 at 640x480
+    //     D = 32: 0.145 / 0.164 at 480x400, 0.151 / 0.161 at 560x400, 0.198 / 0.175 at 640x480
     //   pose: 0.150 / 0.166 at 640x480, 0.251 / 0.243 at 1200x680; D = 32: 0.191 / 0.150 at 640x480
-    const int per_sm = map && factored ? 7 : D == 16 ? 32 : 20;
+    const int per_sm = map && factored ? (D == 16 ? 24 : 16) : D == 16 ? 32 : map ? 24 : 20;
     const int np = prm.bwd_np ? prm.bwd_np
                    : !pr.bwd_warp ? default_bwd_np(D)
                                   : 4 * (int64_t)vt.tile_off[n_views] < (int64_t)kSMs * per_sm ? 1 : 2;

@@ -68,7 +68,7 @@ struct WarpLayout {
     // The contraction runs in up to four chunks of terms so that a lane's running sums fit in
     // its registers (at most 2 CAPS values): the first chunk [0, T1) carries the moments,
     // then [T1, T2), [T2, T3) and [T3, NWT).
-    static constexpr int CAPS = NP == 1 ? 12 : KF ? 28 : 18;
+    static constexpr int CAPS = KF ? 28 : NP == 2 ? 18 : D == 32 ? 20 : 12;
     static constexpr int TC = CAPS / 4 * 4;
     static constexpr int T1 = NWT < (CAPS - 6) / 4 * 4 ? NWT : (CAPS - 6) / 4 * 4;
     static constexpr int T2 = NWT < T1 + TC ? NWT : T1 + TC;
@@ -89,11 +89,14 @@ constexpr int kSlots = 8;
 
 // Resident blocks per SM the register allocation must allow: 16 with two pixels per thread (128
 // registers), except the map mode with the features themselves at D = 32 (whose 19 KB of shared memory
-// allows 11 anyway) and the pose mode with the factored form at D = 32 (12); with one pixel per thread 24 (80
-// registers) in pose mode and 20 or 18 in map mode, where 24 would spill (features themselves, 100k
-// Gaussians at 640x480, D = 16: 0.060 against 0.077 ms).
+// allows 11 anyway) and the pose mode with the factored form at D = 32 (12).  With one pixel per thread,
+// which small images take, 16 as well in map mode, so that the contraction runs in fewer chunks (20 and 18 blocks
+// before: factored form, 0.066 -> 0.060 ms at 64x48, 0.093 -> 0.082 at 640x320; features themselves at D = 32, 0.076
+// -> 0.067 at 320x240), but 20 with the features themselves at D = 16
+// (0.098, 0.101 with 16, at 600x384) and, in pose mode, 24 at D = 16 (0.069, 0.072) and 20 at D = 32 (0.050 with 24,
+// 0.047 at 320x240).
 template <int D, int NP, bool MAP, int KF> constexpr int warp_bwd_min_blocks() {
-    if (NP == 1) return !MAP ? 24 : (D == 32 && KF == 0) ? 18 : 20;
+    if (NP == 1) return !MAP ? (D == 16 ? 24 : 20) : (D == 16 && KF == 0) ? 20 : 16;
     return (D == 32 && (MAP ? KF == 0 : KF > 0)) ? (MAP ? 11 : 12) : 16;
 }
 

@@ -15,9 +15,11 @@ namespace {
 
 // Resident CTAs per SM the register allocation must allow, per feature width and
 // pixels per thread: the blend loop is issue-bound, so warps resident matter
-// more than the few values ptxas would otherwise keep live across the mask flush.
+// more than the few values ptxas would otherwise keep live across the mask flush.  At D = 16 with one
+// pixel per thread four CTAs rather than five (64 registers, 48): with 48 the loads of the two splats
+// evaluated together are taken apart (0.054 -> 0.044 ms at 320x240, 0.067 -> 0.056 at 64x48).
 constexpr int fwd_min_blocks(int D, int NP) {
-    return NP == 1 ? (D == 0 ? 8 : D <= 4 ? 6 : D <= 16 ? 5 : 3) : NP == 2 ? (D <= 16 ? 6 : 4) : 6;
+    return NP == 1 ? (D == 0 ? 8 : D <= 4 ? 6 : D <= 8 ? 5 : D <= 16 ? 4 : 3) : NP == 2 ? (D <= 16 ? 6 : 4) : 6;
 }
 
 // A staged splat is one record of 3 + D / 4 16-byte words: geometry (two), colour and depth, the
@@ -671,13 +673,13 @@ extern "C" gs_status gs_render_fwd(const gs_gaussians *g, const gs_projected *pr
     }
     int np = prm.fwd_np ? prm.fwd_np : default_fwd_np(g->feat_dim);
     // The default at D = 16 and 32 is two pixels per thread, and one where the image has too few tiles for
-    // that: up to one wave of the two-pixel CTAs at D = 16 (six per SM) and two at D = 32 (four per SM) twice
-    // as many warps hide more latency.  Measured, one against two pixels per thread: D = 16: 0.023 / 0.025
-    // ms at 160x120, 0.055 / 0.059 at 320x240, 0.075 / 0.081 at 480x360, but 0.146 / 0.135 (scan) at 640x480
-    // and 0.262 / 0.231 at 1200x680; D = 32: 0.053 / 0.063 at 320x240, 0.148 / 0.163 at 640x480, but 0.114 /
-    // 0.109 at 811x607.  The images do not depend on it.
+    // that: up to two waves of the two-pixel CTAs (six per SM at D = 16, four at D = 32) twice as many warps
+    // hide more latency.  Measured, one against two pixels per thread: D = 16: 0.044 / 0.058 ms at 320x240, 0.068
+    // / 0.084 at 640x480, 0.145 / 0.156 (scan) at 800x600, then 0.103 / 0.098 at 880x600 and 0.237 / 0.218 at
+    // 1200x680; D = 32: 0.053 / 0.063 at 320x240, 0.148 / 0.163 at 640x480, but 0.114 / 0.109 at 811x607.  The
+    // images do not depend on it.
     if (!prm.fwd_np && g->feat_dim >= 16 && prm.fwd_blocks == GS_BWD_BLOCKS_DEFAULT && prm.fwd_batch == kBatch &&
-        vt.tile_off[n_views] <= kSMs * (g->feat_dim == 16 ? 6 : 8))
+        vt.tile_off[n_views] <= kSMs * (g->feat_dim == 16 ? 12 : 8))
         np = 1;
     prm.fwd_group = prm.fwd_blocks == GS_BWD_BLOCKS_GROUP;
     prm.fwd_queue = prm.fwd_blocks == GS_BLOCKS_QUEUE;

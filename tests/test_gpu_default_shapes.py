@@ -22,10 +22,13 @@ def _shape(r, **kw):
     r.prm_c = dataclasses.replace(r.params, **kw).c()
 
 
-# forward: 912 tiles at D = 16, 1216 at D = 32; backward: 266 (map, factored), 1216 (D = 16) or 760 (D = 32)
+# forward: 1824 tiles at D = 16, 1216 at D = 32; backward at D = 16 and 32: 912, 608 (map, factored), 1216, 912 (map,
+# features), 1216, 760 (pose)
 @pytest.mark.parametrize("d,w,h", [(16, 16, 16), (16, 17, 33), (16, 304, 224), (16, 299, 219), (16, 608, 384),
                                    (16, 600, 391), (16, 640, 480), (16, 641, 497), (32, 33, 16), (32, 304, 224),
-                                   (32, 640, 304), (32, 641, 305), (32, 608, 512), (32, 600, 521)])
+                                   (32, 640, 304), (32, 641, 305), (32, 608, 512), (32, 600, 521),
+                                   (16, 912, 512), (16, 900, 529), (16, 601, 390), (32, 608, 256), (32, 601, 255),
+                                   (32, 608, 384), (32, 595, 377)])
 def test_default_shapes_match_the_explicit_ones(d, w, h):
     gs, cam = C.box_case(3000, d, w, h, 0.9 * w)
     field, r = C.gpu_forward(gs, cam, raster.RasterParams(), n_classes=8)

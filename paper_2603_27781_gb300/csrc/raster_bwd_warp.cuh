@@ -87,17 +87,19 @@ template <int V> struct IntC { static constexpr int value = V; };
 // resident blocks (pose mode, 300k scanned Gaussians at 1200x680: 0.241 ms, 0.265 with 16).
 constexpr int kSlots = 8;
 
-// Resident blocks per SM the register allocation must allow: 16 with two pixels per thread (128
-// registers), except the map mode with the features themselves at D = 32 (whose 19 KB of shared memory
-// allows 11 anyway) and the pose mode with the factored form at D = 32 (12).  With one pixel per thread,
-// which small images take, 16 as well in map mode, so that the contraction runs in fewer chunks (20 and 18 blocks
-// before: factored form, 0.066 -> 0.060 ms at 64x48, 0.093 -> 0.082 at 640x320; features themselves at D = 32, 0.076
-// -> 0.067 at 320x240), but 20 with the features themselves at D = 16
-// (0.098, 0.101 with 16, at 600x384) and, in pose mode, 24 at D = 16 (0.069, 0.072) and 20 at D = 32 (0.050 with 24,
-// 0.047 at 320x240).
+// Resident blocks per SM the register allocation must allow.  With two pixels per thread 16 in map mode (128
+// registers), except with the features themselves at D = 32, whose 19 KB of shared memory allow 11
+// anyway; in pose mode 18 at D = 16 (96 registers: 0.243 -> 0.232 ms, 300k scanned Gaussians at 1200x680; 0.240 with
+// 14, 0.237 with 20) and 14 at D = 32 (factored form, 0.151 -> 0.147 ms, 1M Gaussians at 640x480).  With
+// one pixel per thread, which small images take, 16 as well in map mode, so that the contraction runs
+// in fewer chunks (20 and 18 blocks before: factored form, 0.066 -> 0.060 ms at 64x48, 0.093 -> 0.082 at 640x320;
+// features themselves at D = 32, 0.076 -> 0.067 at 320x240), but 20 with the features themselves at D = 16 (0.098 ms,
+// 0.101 with 16, at 600x384) and, in pose mode, 24 at D = 16 (0.069, 0.072) and 20 at D = 32 (0.050 with 24, 0.047 at
+// 320x240).
 template <int D, int NP, bool MAP, int KF> constexpr int warp_bwd_min_blocks() {
     if (NP == 1) return !MAP ? (D == 16 ? 24 : 20) : (D == 16 && KF == 0) ? 20 : 16;
-    return (D == 32 && (MAP ? KF == 0 : KF > 0)) ? (MAP ? 11 : 12) : 16;
+    if (!MAP) return D == 16 ? 18 : 14;
+    return D == 32 && KF == 0 ? 11 : 16;
 }
 
 template <int D, int NP, bool MAP, int KF, typename RT, typename FT>

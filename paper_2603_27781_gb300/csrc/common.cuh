@@ -73,12 +73,6 @@ __device__ __forceinline__ int view_of_tile(const ViewTable &vt, int gt) {
     return v;
 }
 
-__device__ __forceinline__ int view_of_pixel(const ViewTable &vt, int64_t pix) {
-    int v = 0;
-    while (v + 1 < vt.n_views && pix >= vt.pix_off[v + 1]) ++v;
-    return v;
-}
-
 // Loads row-major world->camera rows 0..2, from device poses when given.
 __device__ __forceinline__ void load_pose(const ViewTable &vt, const float *pose_dev, int v,
                                           float R[9], float t[3]) {

@@ -129,7 +129,7 @@ typedef struct {
      * looks at (a test hook: gs_bin_sort then reports GS_ERR_TIMEOUT whenever a
      * radix pass has more than one block of keys: 1,024 visible items per depth
      * pass block up to 2^21 (view, Gaussian) items and 2,048 above, 4,096
-     * instances per tile pass block; and a GS_BLOCKS_RING
+     * instances per tile pass block, 8,192 above 16,384 tiles; and a GS_BLOCKS_RING
      * forward whenever one of its warps has to wait for another). */
     int32_t spin_limit;
     /* Splats the per-tile forward (fwd_blocks GS_BWD_BLOCKS_TILE or

@@ -90,7 +90,6 @@ WsLayout ws_layout(int64_t n, int n_views, int64_t capacity, const ViewTable *vt
     int64_t scan_n = vn > capacity ? vn : capacity;
     int64_t nb1 = (scan_n + 255) / 256 + 1;  // block sums of the 256-item emission blocks (the largest use)
     L.lb_tiles_depth = (int)((vn + depth_sort_tile(vn) - 1) / depth_sort_tile(vn));
-    L.lb_tiles_inst = (int)((capacity + kSortTileInst - 1) / kSortTileInst);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
     L.scan_blocks = take(sizeof(uint32_t) * (size_t)nb1);
@@ -104,7 +103,7 @@ WsLayout ws_layout(int64_t n, int n_views, int64_t capacity, const ViewTable *vt
     L.tkeys_b = take(sizeof(uint32_t) * (size_t)capacity);
     L.tvals_b = take(sizeof(uint32_t) * (size_t)capacity);
     L.hist = take(sizeof(uint32_t) * 8 * 256);
-    L.lookback = take(sizeof(uint32_t) * 256 * ((size_t)4 * L.lb_tiles_depth + (size_t)3 * L.lb_tiles_inst));
+    L.lookback = take(sizeof(uint32_t) * 256 * ((size_t)4 * L.lb_tiles_depth + 3 * (size_t)((capacity + 8191) / 8192)));
     L.tile_counts = take(sizeof(uint32_t) * (vt ? (size_t)vt->tile_off[vt->n_views] : 0));
     L.bin_end = off;
     off = 0;

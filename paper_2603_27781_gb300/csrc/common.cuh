@@ -335,7 +335,7 @@ struct WsLayout {
     size_t dkeys_a, dvals_a, dkeys_b, dvals_b;  // u32 [VN]
     size_t tkeys_a, tkeys_b, tvals_b;           // u32 [capacity]
     size_t hist;          // u32 [8 passes][256]
-    size_t lookback;      // u32 [8 passes][max tiles][256]
+    size_t lookback;      // u32 [4 depth passes][chunks][256], then 768 per 8,192 instances for the tile passes
     size_t tile_counts;   // u32 [total image tiles]: instances per image tile
     size_t bin_end;
     // loss / dsr
@@ -348,7 +348,7 @@ struct WsLayout {
     size_t misc_end;
     size_t total;
     int64_t vn, capacity;
-    int lb_tiles_depth, lb_tiles_inst;
+    int lb_tiles_depth;
 };
 
 constexpr int kLossBlocks = 1024;
@@ -361,7 +361,7 @@ constexpr int64_t kSortSmallItems = (int64_t)1 << 21;
 constexpr int kSortIPTSmall = 4, kSortIPTLarge = 8;  // keys per thread of a depth-sort pass
 inline int depth_sort_tile(int64_t vn) { return kSortThreads * (vn <= kSortSmallItems ? kSortIPTSmall : kSortIPTLarge); }
 constexpr int kSortThreadsInst = 512;   // threads of a tile-sort pass block
-constexpr int kSortIPTInst = 8;         // keys per thread of a tile-sort pass
+constexpr int kSortIPTInst = 8;         // keys per thread of a tile-sort pass (or twice as many)
 constexpr int kSortTileInst = kSortThreadsInst * kSortIPTInst;
 constexpr int kScanIPT = 8;
 constexpr int kScanBlock = 256 * kScanIPT;

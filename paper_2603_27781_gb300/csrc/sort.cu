@@ -13,8 +13,8 @@
 //
 // The digit histograms of every pass are counted by the kernels that write the keys (the
 // compaction for the depth keys, the emission for the tile keys) with shared-memory atomics.
-// Each radix pass is one kernel: a block ranks its keys (1024 or 2048 in a depth pass, 4096 in a tile
-// pass) stably within the block (peer lanes of a digit from one ballot per digit bit + per-warp digit
+// Each radix pass is one kernel: a block ranks its keys (1024 or 2048 in a depth pass, 4096 or 8192 in
+// a tile pass) stably within the block (peer lanes of a digit from one ballot per digit bit + per-warp digit
 // counters), publishes its per-digit
 // counts, finds its global offsets by a chained look-back over earlier blocks,
 // and scatters through shared memory.  Blocks take chunks of keys from an atomic
@@ -87,7 +87,8 @@ struct BinState {
 // First kernel of a binning: zeroes what the call accumulates into (the ranges, the counters, the instance
 // count and status word, the queued forward's work counters, the tile counts, the emission's per-block
 // instance counts, the digit histograms and the look-back flags, the last and largest in 16-byte stores over
-// the whole grid) and counts the visible items of its scan block (grid: at least the count's scan blocks).
+// the whole grid; above kSortSmallItems items without the depth passes' flags) and counts the visible items of
+// its scan block (grid: at least the count's scan blocks).
 __global__ void __launch_bounds__(256) init_reduce_kernel(BinState b, const int32_t *touched, int64_t count,
                                                           uint32_t *block_sums) {
     pdl_wait();     // the previous kernel's results
@@ -189,10 +190,14 @@ __device__ __forceinline__ void hist_flush(uint32_t (*sh)[256], int n_passes, ui
 // Order-preserving compaction of the visible items with their depth keys; also the digit
 // histograms of the depth sort's four passes (no separate pass over the keys), counted over the
 // block's visible keys gathered in shared memory, so that the warps count only visible keys
-// (about a fifth of the items of a frame) in whole rounds of 32.
+// (about a fifth of the items of a frame) in whole rounds of 32.  With lookback, it also clears
+// the four passes' look-back flags, one row of 256 per chunk of visible keys: above kSortSmallItems items, where clearing
+// them for every item there could be costs more than it delays this kernel (32 MB for eight frames of a 2M-Gaussian
+// map: binning 0.860 -> 0.846 ms with the narrower rows of the tile passes; one frame of 1M: 0.138, 0.140 if cleared here).
 __global__ void __launch_bounds__(256) vis_compact_kernel(const int32_t *touched, const float4 *uvdo, int64_t count,
                                                           const uint32_t *block_sums, uint32_t *keys, uint32_t *vals,
-                                                          uint32_t *hist) {
+                                                          uint32_t *hist, const uint32_t *n_vis, uint4 *lookback,
+                                                          int lb_tiles, int chunk) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
     __shared__ uint32_t s_warp[8];
@@ -239,6 +244,11 @@ __global__ void __launch_bounds__(256) vis_compact_kernel(const int32_t *touched
         hist_add(sh, 4, 8, i < tot, i < tot ? s_key[i] : 0u);
     }
     hist_flush(sh, 4, hist);
+    if (!lookback) return;
+    const int64_t row4 = (int64_t)((*n_vis + chunk - 1) / chunk) * 64;  // 16-byte words of a pass
+    for (int p = 0; p < 4; ++p)
+        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < row4; i += (int64_t)gridDim.x * 256)
+            lookback[(int64_t)p * lb_tiles * 64 + i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // ------------------------------------------------------------ instance emission
@@ -342,14 +352,14 @@ struct SortSmem {
 };
 
 // One radix pass over BITS-wide digits, NT threads per block and IPT keys per thread: 256 threads for the
-// depth passes over the visible items, 512 with 8 keys for the tile passes over the instances.
+// depth passes over the visible items, 512 with 8 or 16 keys for the tile passes over the instances.
 // Resident blocks per SM the register allocation must allow: four depth-pass blocks of 8 keys a
-// thread (64 registers), six of 4 (40); three tile-pass blocks (42 registers).  Whole binning in ms with
+// thread (64 registers), six of 4 (40); three tile-pass blocks of 8 (42 registers), two of 16 (64).  Whole binning in ms with
 // tile-pass blocks of 512 x 8 keys at three per SM, 1024 x 8 at two, 512 x 16 at two, 256 x 16 at four: 0.143 / 0.149 /
 // 0.146 / 0.149 (1M Gaussians at 1200x680, 1.7M instances), 0.091 / 0.098 / 0.096 / 0.096 (300k at 811x607),
 // 0.87 / 0.91 / 0.86 / 0.85 (2M, eight keyframes, 22M instances).
 template <int NT, int IPT> constexpr int sort_min_blocks() {
-    return NT == 256 ? (IPT >= 8 ? 4 : 6) : (NT == 512 ? 3 : 2);
+    return NT == 256 ? (IPT >= 8 ? 4 : 6) : (IPT >= 16 ? 2 : 3);
 }
 
 // Lanes of the warp with the same digit (among the lanes in `valid`), by one ballot per bit: a fraction of the
@@ -404,7 +414,7 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
         // an earlier wait gave up (or the count overflowed): this pass's output is not used.  The
         // block still publishes an inclusive prefix (0: never more than the true one, so a block
         // that adds it scatters in bounds) so that no running block waits for it.
-        if (tid < BINS) st_relaxed(lookback + (size_t)tile * 256 + tid, kFlagPre);
+        if (tid < BINS) st_relaxed(lookback + (size_t)tile * BINS + tid, kFlagPre);
         return;
     }
 
@@ -438,7 +448,7 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
     // digits that share their barriers
     const int d = tid;
     uint32_t cnt = 0, hist_d = 0;
-    uint32_t *my = lookback + (size_t)tile * 256 + (d & (BINS - 1));
+    uint32_t *my = lookback + (size_t)tile * BINS + (d & (BINS - 1));
     uint32_t ci = 0, hi = 0;
     if (d < BINS) {
         hist_d = pass_hist[d];
@@ -497,7 +507,7 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
         while (!done && t >= 0) {
             uint32_t w[kWin];
 #pragma unroll
-            for (int i = 0; i < kWin; ++i) w[i] = t - i >= 0 ? ld_relaxed(lookback + (size_t)(t - i) * 256 + d) : 0u;
+            for (int i = 0; i < kWin; ++i) w[i] = t - i >= 0 ? ld_relaxed(lookback + (size_t)(t - i) * BINS + d) : 0u;
 #pragma unroll
             for (int i = 0; i < kWin; ++i) {
                 if (done) continue;
@@ -508,7 +518,7 @@ __global__ void __launch_bounds__(NT, sort_min_blocks<NT, IPT>()) onesweep_kerne
                 }
                 uint32_t vv = w[i];
                 if ((vv & ~kValMask) == 0u) {
-                    const uint32_t *pp = lookback + (size_t)(t - i) * 256 + d;
+                    const uint32_t *pp = lookback + (size_t)(t - i) * BINS + d;
                     int spin = 0;
                     while ((vv & ~kValMask) == 0u && spin < spin_limit) {
                         if (++spin > 64) __nanosleep(64);
@@ -621,7 +631,7 @@ gs_status radix_sort(SortBufs b, const uint32_t *count_ptr, int64_t max_count, i
     uint32_t *ki = b.k0, *vi = b.v0, *ko = b.k1, *vo = b.v1;
     for (int p = 0; p < n_passes; ++p) {
         const gs_status s = launch_pdl(onesweep_kernel<NT, IPT, BITS>, grid, NT, smem, st, ki, vi, ko, vo, count_ptr,
-                                       BITS * p, hist + 256 * p, tile_ctrs + p, lookback + (size_t)p * lb_tiles * 256,
+                                       BITS * p, hist + 256 * p, tile_ctrs + p, lookback + ((size_t)p * lb_tiles << BITS),
                                        status, spin_limit, p == n_passes - 1 ? tile_counts : nullptr, n_tiles, emit_touched,
                                        p == n_passes - 1 ? emit_sums : nullptr, emit_vn);
         if (s) return s;
@@ -732,11 +742,30 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     // Every kernel of the binning is launched with programmatic stream serialization: it is
     // scheduled while its predecessor drains and waits for it (pdl_wait) before reading.
     gs_status s;
-    const int64_t n_lb4 = vn > 0 ? 64 * ((int64_t)4 * L.lb_tiles_depth + (int64_t)3 * L.lb_tiles_inst) : 0;
+    int tile_bits = 1;
+    while (((int64_t)1 << tile_bits) < total_tiles) ++tile_bits;
+    // the fewest passes of at most 8 bits, and digits no wider than those passes need: fewer digits mean
+    // fewer ballots, counters and look-back words per block and longer runs to write (1200x680: two passes
+    // of 6 bits)
+    const int tile_passes = (tile_bits + 7) / 8;
+    const int digit_bits = std::max(5, (tile_bits + tile_passes - 1) / tile_passes);
+    // Chunks of 16 keys a thread where several passes have 8-bit digits (more than 16,384 tiles: large
+    // batches, where they are as fast), of 8 elsewhere: the look-back rows, as wide as the digits, then fit in the
+    // workspace's 768 words per 8,192 instances.
+    const bool wide = digit_bits == 8 && tile_passes > 1;
+    const int lb_tiles = ceil_div(out->capacity, wide ? 2 * kSortTileInst : kSortTileInst);
+    uint32_t *tile_lookback = lookback + (size_t)4 * L.lb_tiles_depth * 256;
+    // look-back flags that the first kernel clears: of all passes (the depth passes' come first), or above
+    // kSortSmallItems items of the tile passes, the compaction clearing the others
+    const bool clear_first = vn <= kSortSmallItems;
+    const int64_t n_lb4 = vn > 0 ? (((int64_t)tile_passes * lb_tiles << digit_bits) / 4 +
+                                    (clear_first ? 4 * (int64_t)L.lb_tiles_depth * 64 : 0))
+                                 : 0;
     const int64_t nbe = ceil_div(vn, kEmitBlock);  // emission blocks
     const int nb = ceil_div(vn, kScanBlock);       // scan blocks
     const int init_grid = std::max<int>({1, nb, (int)std::min<int64_t>((n_lb4 + 255) / 256, kSMs * 8)});
-    const BinState state{out->ranges, counters, tile_counts, emit_sums, hist, out->queue, reinterpret_cast<uint4 *>(lookback),
+    const BinState state{out->ranges, counters, tile_counts, emit_sums, hist, out->queue,
+                         reinterpret_cast<uint4 *>(clear_first ? lookback : tile_lookback),
                          2 * total_tiles, total_tiles, nbe + 1, n_lb4, out->n_inst, out->status};
     // 1. the call's state; the visible items of every scan block
     if ((s = launch_pdl(init_reduce_kernel, init_grid, 256, 0, st, state, proj->tiles_touched, vn, block_sums))) return s;
@@ -752,7 +781,9 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
                         (int)CTR_NVIS, -1, (int64_t)0, nullptr, nullptr)))
         return s;
     if ((s = launch_pdl(vis_compact_kernel, nb, 256, 0, st, proj->tiles_touched, uvdo, vn, block_sums, dk_a, dv_a,
-                        hist)))
+                        hist, counters + CTR_NVIS,
+                        clear_first ? (uint4 *)nullptr : reinterpret_cast<uint4 *>(lookback), L.lb_tiles_depth,
+                        depth_sort_tile(vn))))
         return s;
 
     // 2. stable sort of the visible items by depth (4 passes: result in dk_a/dv_a); the last pass
@@ -768,13 +799,6 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     const uint32_t *sorted_items = dv_a;
 
     // 3. emit instances in depth order; instance count -> n_inst (clamped copy for the sort)
-    int tile_bits = 1;
-    while (((int64_t)1 << tile_bits) < total_tiles) ++tile_bits;
-    // the fewest passes of at most 8 bits, and digits no wider than those passes need: fewer digits mean
-    // fewer ballots, counters and look-back words per block and longer runs to write (1200x680: two passes
-    // of 6 bits)
-    const int tile_passes = (tile_bits + 7) / 8;
-    const int digit_bits = std::max(5, (tile_bits + tile_passes - 1) / tile_passes);
     uint32_t *tk_a = reinterpret_cast<uint32_t *>(w + L.tkeys_a), *tk_b = reinterpret_cast<uint32_t *>(w + L.tkeys_b);
     uint32_t *tv_b = reinterpret_cast<uint32_t *>(w + L.tvals_b);
     // the emitted values go where the final pass must not land: out->vals ends the sort
@@ -790,16 +814,18 @@ extern "C" gs_status gs_bin_sort(int64_t n, const gs_projected *proj, const gs_c
     if (out->capacity == 0) return write_ranges_order(tile_counts, out, total_tiles, st);
 
     // 4. stable sort of the instances by tile id
-    auto tile_sort = [&](auto bits) {
-        return radix_sort<kSortThreadsInst, kSortIPTInst, decltype(bits)::value>(
+    auto tile_sort = [&](auto ipt, auto bits) {
+        return radix_sort<kSortThreadsInst, decltype(ipt)::value, decltype(bits)::value>(
             {tk_a, emit_vals, tk_b, other_vals}, counters + CTR_M, out->capacity, tile_passes, hist + 4 * 256,
-            lookback + (size_t)4 * L.lb_tiles_depth * 256, L.lb_tiles_inst, counters + CTR_TILE + 4, out->status,
-            prm.spin_limit, st, tile_counts, (uint32_t)total_tiles);
+            tile_lookback, lb_tiles, counters + CTR_TILE + 4, out->status, prm.spin_limit, st, tile_counts,
+            (uint32_t)total_tiles);
     };
-    s = digit_bits == 5   ? tile_sort(std::integral_constant<int, 5>())
-        : digit_bits == 6 ? tile_sort(std::integral_constant<int, 6>())
-        : digit_bits == 7 ? tile_sort(std::integral_constant<int, 7>())
-                          : tile_sort(std::integral_constant<int, 8>());
+    constexpr std::integral_constant<int, kSortIPTInst> keys8;
+    s = digit_bits == 5   ? tile_sort(keys8, std::integral_constant<int, 5>())
+        : digit_bits == 6 ? tile_sort(keys8, std::integral_constant<int, 6>())
+        : digit_bits == 7 ? tile_sort(keys8, std::integral_constant<int, 7>())
+        : !wide           ? tile_sort(keys8, std::integral_constant<int, 8>())
+                          : tile_sort(std::integral_constant<int, 2 * kSortIPTInst>(), std::integral_constant<int, 8>());
     if (s) return s;
     const uint32_t *sorted_tiles = (tile_passes % 2 == 0) ? tk_a : tk_b;
 

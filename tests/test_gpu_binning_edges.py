@@ -78,3 +78,18 @@ def test_more_than_one_wave_of_chunks():
     _, r = C.gpu_forward(gs, cams, raster.RasterParams())
     assert r.instances() > 4096 * 152 * 3 * 2
     _check(r, gs, cams)
+
+
+# more than 2^21 (view, Gaussian) items: chunks of 2,048 items and their look-back flags cleared by the compaction, few and
+# many of them visible, on buffers that an earlier call has filled
+@pytest.mark.parametrize("facing", [True, False])
+def test_many_items_of_which_few_are_visible(facing):
+    gs, cam = C.box_case(270_000, 4, 64, 48, 60.0)
+    away = synth.camera(64, 48, 60.0, T_cw=np.diag([-1.0, 1.0, -1.0, 1.0]))
+    cams = [cam] * 8 if facing else [away, cam] + [away] * 6
+    gs.log_scales[:] -= 3.0   # small splats: the instances stay few
+    field, r = C.gpu_forward(gs, cams, raster.RasterParams())
+    _check(r, gs, cams)
+    r.project(field)
+    r.bin_sort(want_keys=True)
+    _check(r, gs, cams)

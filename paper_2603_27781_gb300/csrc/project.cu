@@ -27,15 +27,14 @@ struct Shape {
     bool ok;
 };
 
-__device__ __forceinline__ void load_shape(const float *quats, const float *log_scales, uint32_t g, Shape &sh) {
-    float4 q = reinterpret_cast<const float4 *>(quats)[g];
+__device__ __forceinline__ void make_shape(float4 q, const float (&log_scale)[3], Shape &sh) {
     sh.qn = sqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
     sh.ok = sh.qn > 0.f;
     float inv = sh.ok ? 1.f / sh.qn : 0.f;
     sh.qh[0] = q.x * inv; sh.qh[1] = q.y * inv; sh.qh[2] = q.z * inv; sh.qh[3] = q.w * inv;
     quat_rot(sh.qh, sh.Rq);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) sh.s[c] = expf(log_scales[3 * (size_t)g + c]);
+    for (int c = 0; c < 3; ++c) sh.s[c] = expf(log_scale[c]);
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -47,6 +46,11 @@ __device__ __forceinline__ void load_shape(const float *quats, const float *log_
     sh.Sig.m[3] = M[3] * M[3] + M[4] * M[4] + M[5] * M[5];
     sh.Sig.m[4] = M[3] * M[6] + M[4] * M[7] + M[5] * M[8];
     sh.Sig.m[5] = M[6] * M[6] + M[7] * M[7] + M[8] * M[8];
+}
+
+__device__ __forceinline__ void load_shape(const float *quats, const float *log_scales, uint32_t g, Shape &sh) {
+    const float l[3] = {log_scales[3 * (size_t)g], log_scales[3 * (size_t)g + 1], log_scales[3 * (size_t)g + 2]};
+    make_shape(reinterpret_cast<const float4 *>(quats)[g], l, sh);
 }
 
 __device__ __forceinline__ float sym(const Cov3 &c, int r, int k) {
@@ -135,6 +139,43 @@ __device__ __forceinline__ void project_geo(const float mu[3], const Shape &sh, 
     o.ok = isfinite(o.u) && isfinite(o.v) && isfinite(o.A) && isfinite(o.B) && isfinite(o.C);
 }
 
+// Arrays that the projection writes.
+struct ProjOut {
+    float4 *uvdo;
+    float2 *uv_lo;
+    float4 *conic;
+    int32_t *touched;
+};
+
+// The record of one (view, Gaussian) item of opacity o from its geometry.
+__device__ __forceinline__ void write_item(const ViewTable &vt, const Params &prm, int v, const Geo &ge, float o, uint32_t item,
+                                           const ProjOut &out) {
+    float4 rec = make_float4(0.f, 0.f, ge.p[2], o);
+    float2 lo = make_float2(0.f, 0.f);
+    float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
+    int tt = 0;
+    if (ge.ok) {
+        float mid = 0.5f * (ge.a + ge.c);
+        float det = ge.a * ge.c - ge.b * ge.b;
+        float lmax = mid + sqrtf(fmaxf(mid * mid - det, 0.f));
+        float rr = fminf(prm.radius_sigma * sqrtf(lmax), 16777216.f);
+        int r = (int)ceilf(rr);
+        if (r > 0) {
+            int x0, y0, x1, y1;
+            tile_rect(ge.u, ge.v, r, vt.TX[v], vt.TY[v], x0, y0, x1, y1);
+            tt = (x1 - x0) * (y1 - y0);
+        }
+        rec.x = ge.u;
+        rec.y = ge.v;
+        lo = make_float2(ge.ulo, ge.vlo);
+        cn = make_float4(ge.A, ge.B, ge.C, (float)r);
+    }
+    out.uvdo[item] = rec;
+    out.uv_lo[item] = lo;
+    out.conic[item] = cn;
+    out.touched[item] = tt;
+}
+
 // A thread projects its Gaussian into views [blockIdx.y * per, (blockIdx.y + 1) * per): the parameters are
 // read, activated and turned into the 3D covariance once for all of them.  Bound by instruction issue
 // (84 % of cycles; the compensated centre, the activation and the covariance products).
@@ -143,9 +184,7 @@ __global__ void __launch_bounds__(256, 6) project_fwd_kernel(ViewTable vt, Param
                                                           const float *__restrict__ quats,
                                                           const float *__restrict__ log_scales,
                                                           const float *__restrict__ logits,
-                                                          const float *__restrict__ pose_dev, float4 *__restrict__ uvdo,
-                                                          float2 *__restrict__ uv_lo, float4 *__restrict__ conic,
-                                                          int32_t *__restrict__ touched) {
+                                                          const float *__restrict__ pose_dev, ProjOut out) {
     pdl_wait();     // the previous kernel's results
     pdl_trigger();  // the next kernel may be scheduled now
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -162,31 +201,90 @@ __global__ void __launch_bounds__(256, 6) project_fwd_kernel(ViewTable vt, Param
         load_pose(vt, pose_dev, v, R, t);
         Geo ge;
         project_geo(mu, sh, R, t, vt, v, prm, ge, true);
-        float4 rec = make_float4(0.f, 0.f, ge.p[2], o);
-        float2 lo = make_float2(0.f, 0.f);
-        float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
-        int tt = 0;
-        if (ge.ok) {
-            float mid = 0.5f * (ge.a + ge.c);
-            float det = ge.a * ge.c - ge.b * ge.b;
-            float lmax = mid + sqrtf(fmaxf(mid * mid - det, 0.f));
-            float rr = fminf(prm.radius_sigma * sqrtf(lmax), 16777216.f);
-            int r = (int)ceilf(rr);
-            if (r > 0) {
-                int x0, y0, x1, y1;
-                tile_rect(ge.u, ge.v, r, vt.TX[v], vt.TY[v], x0, y0, x1, y1);
-                tt = (x1 - x0) * (y1 - y0);
-            }
-            rec.x = ge.u;
-            rec.y = ge.v;
-            lo = make_float2(ge.ulo, ge.vlo);
-            cn = make_float4(ge.A, ge.B, ge.C, (float)r);
-        }
-        uvdo[item] = rec;
-        uv_lo[item] = lo;
-        conic[item] = cn;
-        touched[item] = tt;
+        write_item(vt, prm, v, ge, o, item, out);
     }
+}
+
+// One view, 256 consecutive Gaussians a block.  Of a map around the camera a good part lies behind it, spread over
+// the index space, and the kernel is bound by instruction issue: each thread tests its own Gaussian's depth and
+// writes the empty record of one behind, and the block's first warps project the listed others in full
+// warps, from parameters that were loaded by their own threads ahead of the test (a block with none behind
+// makes no list).  1M Gaussians around the camera: 0.0230 -> 0.0174 ms, bit-identical; 850k all in front of it: 0.0192,
+// 0.0196.  With several views, whose parameters and covariance one thread shares, the lists gained nothing
+// (1M in six views: 0.093 ms either way).
+constexpr int kProjThreads = 256;
+__global__ void __launch_bounds__(kProjThreads, 6) project_fwd_one_kernel(ViewTable vt, Params prm, uint32_t n,
+                                                                          const float *__restrict__ means,
+                                                                          const float *__restrict__ quats,
+                                                                          const float *__restrict__ log_scales,
+                                                                          const float *__restrict__ logits,
+                                                                          const float *__restrict__ pose_dev, ProjOut out) {
+    pdl_wait();     // the previous kernel's results
+    pdl_trigger();  // the next kernel may be scheduled now
+    constexpr int W = kProjThreads / 32, v = 0;
+    __shared__ float4 s_q[kProjThreads];
+    __shared__ float s_ls[3][kProjThreads], s_mu[3][kProjThreads], s_logit[kProjThreads];
+    __shared__ uint8_t s_list[kProjThreads];
+    __shared__ int s_cnt[W];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t g0 = blockIdx.x * kProjThreads, g = g0 + tid;
+    float R[9], t[3], mu[3], ls[3], logit = 0.f;
+    float4 q;
+    bool front = false;
+    if (g < n) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            mu[k] = means[3 * (size_t)g + k];
+            ls[k] = log_scales[3 * (size_t)g + k];
+        }
+        logit = logits[g];
+        q = reinterpret_cast<const float4 *>(quats)[g];
+    }
+    load_pose(vt, pose_dev, v, R, t);
+    if (g < n) {
+        // the depth as project_geo forms it
+        const float z = __fmaf_rn(R[6], mu[0], __fmaf_rn(R[7], mu[1], __fmaf_rn(R[8], mu[2], t[2])));
+        front = z > prm.z_near;
+        if (front) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                s_mu[k][tid] = mu[k];
+                s_ls[k][tid] = ls[k];
+            }
+            s_logit[tid] = logit;
+            s_q[tid] = q;
+        } else {
+            out.uvdo[g] = make_float4(0.f, 0.f, z, 1.f / (1.f + expf(-logit)));
+            out.uv_lo[g] = make_float2(0.f, 0.f);
+            out.conic[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+            out.touched[g] = 0;
+        }
+    }
+    const uint32_t bal = __ballot_sync(0xffffffffu, front);
+    if (lane == 0) s_cnt[w] = __popc(bal);
+    const int total = __syncthreads_count(front);
+    int l = tid;
+    if (total < kProjThreads) {
+        if (front) {
+            int at = __popc(bal & lanemask_lt());
+#pragma unroll
+            for (int i = 0; i < W; ++i) at += i < w ? s_cnt[i] : 0;
+            s_list[at] = (uint8_t)tid;
+        }
+        __syncthreads();
+        if (tid >= total) return;
+        l = s_list[tid];
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        mu[k] = s_mu[k][l];
+        ls[k] = s_ls[k][l];
+    }
+    Shape sh;
+    make_shape(s_q[l], ls, sh);
+    Geo ge;
+    project_geo(mu, sh, R, t, vt, v, prm, ge, true);
+    write_item(vt, prm, v, ge, 1.f / (1.f + expf(-s_logit[l])), g0 + l, out);
 }
 
 // Gradients of one Gaussian collected over the views: its mean, Sigma (trace form) and activated opacity.
@@ -445,11 +543,14 @@ extern "C" gs_status gs_project(const gs_gaussians *g, const gs_camera *cams, in
     const int64_t threads = 2 * (int64_t)kSMs * 2048;
     const int groups = (int)std::min<int64_t>(n_views, (threads + g->n - 1) / g->n);
     const int per = (n_views + groups - 1) / groups;
-    dim3 grid(ceil_div(g->n, 256), (n_views + per - 1) / per);
+    const ProjOut o{reinterpret_cast<float4 *>(out->uvdo), reinterpret_cast<float2 *>(out->uv_lo),
+                    reinterpret_cast<float4 *>(out->conic), out->tiles_touched};
+    if (n_views == 1)
+        return launch_pdl(project_fwd_one_kernel, ceil_div(g->n, kProjThreads), kProjThreads, 0, (cudaStream_t)stream, vt, prm,
+                          (uint32_t)g->n, g->means, g->quats, g->log_scales, g->opacity_logits, pose_dev, o);
+    const dim3 grid(ceil_div(g->n, 256), (n_views + per - 1) / per);
     return launch_pdl(project_fwd_kernel, grid, 256, 0, (cudaStream_t)stream, vt, prm, (uint32_t)g->n, per, g->means, g->quats,
-                      g->log_scales, g->opacity_logits, pose_dev, reinterpret_cast<float4 *>(out->uvdo),
-                      reinterpret_cast<float2 *>(out->uv_lo), reinterpret_cast<float4 *>(out->conic),
-                      out->tiles_touched);
+                      g->log_scales, g->opacity_logits, pose_dev, o);
 }
 
 extern "C" gs_status gs_project_bwd(const gs_gaussians *g, const gs_camera *cams, int n_views, const float *pose_dev,

@@ -89,21 +89,6 @@ __device__ __forceinline__ SplatGeo make_geo(float4 a, float2 lo, float4 c) {
     return s;
 }
 
-// Half extents (x, y) of the region where the splat can reach alpha >= alpha_min:
-// o exp(-q/2) >= alpha_min  <=>  q <= 2 ln(o / alpha_min), and the ellipse
-// x^T Sigma^-1 x <= qmax spans +-sqrt(qmax Sigma_xx) in x.  Widened by 0.1% and
-// 0.01 px so that f32 rounding never culls a pixel the evaluation would blend;
-// infinite (no culling) when alpha_min is 0.
-__device__ __forceinline__ float2 splat_extent(float4 c, float o, float alpha_min) {
-    if (!(alpha_min > 0.f)) return make_float2(INFINITY, INFINITY);
-    if (!(o > alpha_min)) return make_float2(-1.f, -1.f);
-    const float qmax = 2.f * logf(o / alpha_min);
-    const float det = c.x * c.z - c.y * c.y;
-    if (!(det > 0.f)) return make_float2(INFINITY, INFINITY);
-    const float sxx = c.z / det, syy = c.x / det;
-    return make_float2(sqrtf(qmax * sxx) * 1.001f + 0.01f, sqrtf(qmax * syy) * 1.001f + 0.01f);
-}
-
 // Checked build (compiled with GS_CHECKS=1): the indices a blend kernel takes from the
 // binning and the forward images are verified before use.  A tile's instance range must lie
 // within the binning's capacity and a staged item must be one of its view's Gaussians; a
@@ -143,12 +128,6 @@ __device__ __forceinline__ int checked_last(uint32_t start, const uint32_t *rang
     return last;
 }
 
-// Whether a splat centred at (u, v) with extent e can reach the warp's pixel box
-// (pixel centres from (bx0 + 0.5, by0 + 0.5), bw x bh of them).
-__device__ __forceinline__ bool reaches_box(float u, float v, float2 e, float bcx, float bcy, float hx, float hy) {
-    return fabsf(u - bcx) <= e.x + hx && fabsf(v - bcy) <= e.y + hy;
-}
-
 // The splat's constants for reaches_box_exact: the edge optima rx = -qb / (2 qc), ry = -qb /
 // (2 qa) and the exponent threshold log2(alpha_min / o) (-inf when alpha_min is 0).
 __device__ __forceinline__ float4 ellipse_cull(const SplatGeo &s, float alpha_min) {
@@ -157,8 +136,9 @@ __device__ __forceinline__ float4 ellipse_cull(const SplatGeo &s, float alpha_mi
 
 // Whether any point of the box of pixel centres [bcx - hx, bcx + hx] x [bcy - hy, bcy + hy]
 // can have alpha >= alpha_min, i.e. exponent p(x, y) = qa x^2 + qb x y + qc y^2 >= log2(alpha_min
-// / o) with (x, y) relative to the centre: the exact ellipse against the box, where the
-// extent test bounds the ellipse by its rectangle.  p is concave with its maximum 0 at the
+// / o) with (x, y) relative to the centre: the exact ellipse against the box.  (The ellipse's
+// bounding rectangle, from the conic's determinant in f32, is no bound for long thin splats at an
+// angle: at 1000 x 0.7 px sigma it misses blended pixels of two splats in three.)  p is concave with its maximum 0 at the
 // centre; with the centre outside the box its maximum over the box lies on an edge, on the
 // vertical edge x = xe at y = clamp(rx xe) and on the horizontal edge y = ye at
 // x = clamp(ry ye).  Conservative: the box is widened by 0.01 px (the centre's low part and the

@@ -49,13 +49,14 @@ constexpr int walk_splats(int NP) { return NP == 2 ? 4 : NP == 1 ? 2 : 1; }
 // The kernel is bound by instruction issue (74 % of cycles at D = 16) and by the latency of the
 // staging between its barriers.  One base address per record, packed multiply-adds and the exact
 // ellipse test alone (the rectangle test before it cost a logarithm, two roots and two divisions per
-// staged splat and culled almost nothing more) took the forward from 0.266 to 0.246 ms (room, 1M
-// Gaussians, D = 16, 1200x680), 0.230 to 0.190 ms (1M, D = 32, 640x480), 4.33 to 3.26 ms (2M, D = 32,
-// 16-bit storage, 8 keyframes) and 0.107 to 0.075 ms (300k, D = 8, 811x607), bit-identical.  Measured
-// and slower: the next batch's records copied (cp.async) into a second buffer while the current one
-// is walked (0.339 ms with 128-splat batches, 0.282 with 64: the second buffer takes the L1 that
-// serves the gathers of neighbouring tiles), and the box tests done once by the staging thread for
-// all four warps (0.262 against 0.237 ms: they then sit between the loads and the barrier).
+// staged splat and culled little more, blended pixels of long thin splats among it) took the forward
+// from 0.266 to 0.246 ms (room, 1M Gaussians, D = 16, 1200x680), 0.230 to 0.190 ms (1M, D = 32, 640x480),
+// 4.33 to 3.26 ms (2M, D = 32, 16-bit storage, 8 keyframes) and 0.107 to 0.075 ms (300k, D = 8,
+// 811x607), with the same images on these scenes.  Measured and slower: the next batch's records copied
+// (cp.async) into a second buffer while the current one is walked (0.339 ms with 128-splat batches,
+// 0.282 with 64: the second buffer takes the L1 that serves the gathers of neighbouring tiles), and the
+// box tests done once by the staging thread for all four warps (0.262 against 0.237 ms: they then sit
+// between the loads and the barrier).
 template <int D, int NP>
 struct BlendPixels {
     using SH = Shape<NP, true>;  // horizontal pixel pairs

@@ -60,6 +60,13 @@ __device__ __forceinline__ void load_halo(const float *const (&src)[N], int W, i
     }
 }
 
+// sum += x, with what the f32 addition rounds away added to lo (an infinite sum stays one).
+__device__ __forceinline__ void add_exact(float x, float &sum, float &lo) {
+    float e;
+    two_sum(sum, x, sum, e);
+    lo += isfinite(e) ? e : 0.f;
+}
+
 __global__ void __launch_bounds__(kSThreads) ssim_fwd_kernel(ViewTable vt, SsimTable t, const float *rgb,
                                                              const float *trgb, int64_t P, float *maps,
                                                              double *part) {
@@ -68,7 +75,7 @@ __global__ void __launch_bounds__(kSThreads) ssim_fwd_kernel(ViewTable vt, SsimT
     __shared__ float2 s_xy[kIH][kIW + 1];
     __shared__ float2 s_m[kIH][kSW + 1], s_q[kIH][kSW + 1];  // row sums of (x, y), (x^2, y^2) and x y
     __shared__ float s_c[kIH][kSW + 1];
-    __shared__ float s_sum[kSThreads];
+    __shared__ float s_sum[2][kSThreads];
     int v, ch, x0, y0;
     locate(vt, t, v, ch, x0, y0);
     const int W = vt.W[v], H = vt.H[v], lane = threadIdx.x & 31, o0 = threadIdx.x / 32 * kOut;
@@ -108,7 +115,7 @@ __global__ void __launch_bounds__(kSThreads) ssim_fwd_kernel(ViewTable vt, SsimT
     constexpr float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
     const int64_t Pv = (int64_t)W * H;
     float2 m[kOut], q[kOut];
-    float c[kOut], ssum = 0.f;
+    float c[kOut], ssum = 0.f, slo = 0.f;  // the thread's sum of S and what its additions rounded away
 #pragma unroll
     for (int j = 0; j < kOut; ++j) {
         m[j] = q[j] = make_float2(0.f, 0.f);
@@ -146,15 +153,21 @@ __global__ void __launch_bounds__(kSThreads) ssim_fwd_kernel(ViewTable vt, SsimT
         maps[mb + o] = dS_dmx - 2.f * mx * dS_dsx - my * dS_dsxy;
         maps[mb + Pv + o] = dS_dsx;
         maps[mb + 2 * Pv + o] = dS_dsxy;
-        ssum += S;
+        add_exact(S, ssum, slo);
     }
-    // the tile's sum in f64 by one warp (f64 additions are slow: see the loss's block sums)
-    s_sum[threadIdx.x] = ssum;
+    // the tile's sum by one warp, in f64 at the end (f64 additions are slow, see the loss's block sums; f32
+    // sums of values near 1 alone would round away what 1 - SSIM is made of)
+    s_sum[0][threadIdx.x] = ssum;
+    s_sum[1][threadIdx.x] = slo;
     __syncthreads();
     if (threadIdx.x >= 32) return;
-    double tot = 0.0;
+    ssum = slo = 0.f;
 #pragma unroll
-    for (int i = 0; i < kSThreads / 32; ++i) tot += (double)s_sum[i * 32 + lane];
+    for (int i = 0; i < kSThreads / 32; ++i) {
+        add_exact(s_sum[0][i * 32 + lane], ssum, slo);
+        slo += s_sum[1][i * 32 + lane];
+    }
+    double tot = (double)ssum + (double)slo;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     if (lane == 0) {

@@ -67,7 +67,8 @@ __device__ __forceinline__ void add_exact(float x, float &sum, float &lo) {
     lo += isfinite(e) ? e : 0.f;
 }
 
-__global__ void __launch_bounds__(kSThreads) ssim_fwd_kernel(ViewTable vt, SsimTable t, const float *rgb,
+// Five resident blocks per SM (48 registers), as many as its 44 KB of shared memory allow.
+__global__ void __launch_bounds__(kSThreads, 5) ssim_fwd_kernel(ViewTable vt, SsimTable t, const float *rgb,
                                                              const float *trgb, int64_t P, float *maps,
                                                              double *part) {
     pdl_wait();     // the previous kernel's results

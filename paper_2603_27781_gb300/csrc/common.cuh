@@ -234,13 +234,15 @@ template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16
 }
 
 // Exact tile rectangle of a splat (half-open, in tiles): floor((u - r)/16) is
-// floordiv(floor(u) - r, 16) because r is an integer.  In 32 bits: r is at most 2^24 and an image at most 2^15
-// wide, so a centre beyond 2^26 (and one that is not a number, taken as -2^26) lies on the same side of every
-// tile as 2^26 does.
+// floordiv(floor(u) - r, 16) because r is an integer.  In 32 bits: centres and radii are taken within 2^30,
+// where their sums fit (the projection's radii are at most 2^24, those of a caller's own records may be
+// larger).  An image is at most 2^15 wide, so a centre beyond 2^30 (and one that is not a number, taken as
+// -2^30) lies outside it by more than any smaller radius.
 __device__ __forceinline__ void tile_rect(float u, float v, int r, int TX, int TY, int &x0, int &y0,
                                           int &x1, int &y1) {
-    const float lim = 67108864.0f;  // 2^26
+    const float lim = 1073741824.0f;  // 2^30
     const int iu = (int)fminf(fmaxf(floorf(u), -lim), lim), iv = (int)fminf(fmaxf(floorf(v), -lim), lim);
+    r = min(r, (1 << 30) - 1);
     auto cl = [](int a, int hi) { return min(max(a, 0), hi); };
     static_assert(kTile == 16, "a tile is 2^4 pixels");
     x0 = cl((iu - r) >> 4, TX);

@@ -87,12 +87,22 @@ def _stream(stream=None):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+def _copy_all(dst, src):
+    """dst[i].copy_(src[i]) for all i, by one launch where they are dense and of one type (a copy each
+    costs 7 us of host time).  Forward-mode differentiation has no rule for the joint copy and
+    refuses it before anything is copied: then one by one."""
+    try:
+        torch._foreach_copy_(dst, src)
+    except NotImplementedError:
+        for d, s in zip(dst, src):
+            d.copy_(s)
+
+
 def _copies(tensors):
-    """Contiguous copies of a list of tensors by one launch where they are dense and of one type (a
-    clone each costs 7 us of host time and a copy of its own on the device)."""
+    """Contiguous copies of a list of tensors, by one launch (a clone each is a copy of its own on the device)."""
     out = [torch.empty(t.shape, dtype=t.dtype, device=t.device) for t in tensors]
     with torch.no_grad():
-        torch._foreach_copy_(out, tensors)
+        _copy_all(out, tensors)
     return out
 
 
@@ -553,7 +563,7 @@ def expand(r: "Renderer", field: Field, targets, feat_init: torch.Tensor, tau_un
         for t, o in zip(new, old):      # the joint copy has no derivative
             t[:n].copy_(o)
     else:
-        torch._foreach_copy_([t[:n] for t in new], old)
+        _copy_all([t[:n] for t in new], old)
     out = Field(*new)
     fm = L.gs_field_mut(n + n_max, D, _p(out.means), _p(out.quats), _p(out.log_scales), _p(out.opacity_logits),
                         _p(out.rgb), _p(out.feat) if D else None)
@@ -679,7 +689,7 @@ class RasterizeSG(torch.autograd.Function):
         given = [(b, g) for b, g in bufs if g is not None]
         if given:
             with torch.no_grad():       # also under create_graph: nothing here has a second derivative
-                torch._foreach_copy_([b for b, _ in given], [g for _, g in given])
+                _copy_all([b for b, _ in given], [g for _, g in given])
         for b, g in bufs:
             if g is None:
                 b.zero_()

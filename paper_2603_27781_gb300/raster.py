@@ -550,7 +550,8 @@ def expand(r: "Renderer", field: Field, targets, feat_init: torch.Tensor, tau_un
     source pixels, the number of unobserved pixels, the status word: GS_ERR_CAPACITY when that
     number exceeds n_max and only the first n_max were added).  feat_init [n_max, D] holds the
     new Gaussians' features (the caller draws them).  Reads the count back to the host (the
-    field's size sets every later launch)."""
+    field's size sets every later launch).  With `stream`, the library's part runs there, after what the
+    current stream holds; the current stream waits for it, so the results are used as usual."""
     if field.rgb.dtype != torch.float32 or field.feat.dtype != torch.float32:
         raise ValueError("expansion appends to f32 parameter storage")
     n, D = field.n, field.feat_dim
@@ -573,9 +574,13 @@ def expand(r: "Renderer", field: Field, targets, feat_init: torch.Tensor, tau_un
     src = torch.empty(max(n_max, 1), dtype=torch.int64, device=dev)
     tc = L.gs_targets(_p(targets["rgb"]), _p(targets["depth"]), _p(targets["label"]))
     fi = feat_init.contiguous().to(torch.float32)
+    if stream is not None:              # it reads the copies made on the current stream
+        stream.wait_stream(torch.cuda.current_stream())
     L.check("gs_expand", L.gs_expand(r.cams_c, r.n_views, ctypes.byref(r.images_c()), ctypes.byref(tc), tau_unobs,
                                      _p(fi) if D else None, n, ctypes.byref(fm), _p(result), _p(src),
                                      _p(result[2:]), _p(r.ws), r.ws.numel(), _stream(stream)))
+    if stream is not None:              # the result is read, and the memory given back, on the current one
+        torch.cuda.current_stream().wait_stream(stream)
     lo, hi, status = result.tolist()
     total = hi << 32 | (lo & 0xffffffff)
     k = min(total, n_max)

@@ -216,8 +216,8 @@ struct LossGrid {
 //    The sums reach the block's shared ones once, at the end.
 // Loss step (this kernel and the finish), before and now: 0.054 -> 0.047 ms (D = 16, K = 8, 1200x680),
 // 0.433 -> 0.25 (D = 32, K = 8, eight keyframes of two sizes), 0.167 -> 0.096 (D = 16, K = 20, 1200x680, with
-// the features' gradient).  Two pixels a thread where 128 registers hold them without spilling (K = 20:
-// 0.101 with two, 0.096 with one).
+// the features' gradient).  Two pixels a thread where 128 registers hold them with at most 8 bytes
+// spilled (D = 16, K = 8); K = 20: 0.101 with two, 0.096 with one.
 template <int D, int KC>
 struct LossShape {
     static constexpr int NT = 128;                        // keeps the static shared memory < 48 KB

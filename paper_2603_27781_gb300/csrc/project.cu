@@ -405,6 +405,15 @@ __device__ __forceinline__ void write_gauss_grads(const Shape &sh, const GaussSu
     o.logits[g] = op * (1.f - op) * a.dop;
 }
 
+// A Gaussian that no splat sum belongs to: zeros, whatever its parameters (an overflowing scale times a zero sum
+// would not be one).
+__device__ __forceinline__ void write_no_grads(uint32_t g, const BwdOut &o) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) o.means[3 * (size_t)g + k] = o.log_scales[3 * (size_t)g + k] = 0.f;
+    reinterpret_cast<float4 *>(o.quats)[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+    o.logits[g] = 0.f;
+}
+
 // One view: the Gaussians are walked by warps, SPAN at a time.  Most of a map is out of a frame (82 % of the room at
 // 1200x680) and has zero sums, spread over the index space: with a Gaussian per lane nearly every warp ran the
 // whole chain for a fifth of its lanes.  A warp instead reads the splat sums of its span (coalesced),
@@ -442,12 +451,7 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 6) project_bwd_one_kernel(
                 out.rgb[3 * (size_t)g] = cr.x;
                 out.rgb[3 * (size_t)g + 1] = cr.y;
                 out.rgb[3 * (size_t)g + 2] = cr.z;
-                if (!any) {
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) out.means[3 * (size_t)g + k] = out.log_scales[3 * (size_t)g + k] = 0.f;
-                    reinterpret_cast<float4 *>(out.quats)[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    out.logits[g] = 0.f;
-                }
+                if (!any) write_no_grads(g, out);
             }
             if (pose && !any) {
 #pragma unroll
@@ -497,19 +501,23 @@ __global__ void __launch_bounds__(128, 6) project_bwd_kernel(ViewTable vt, Param
     load_shape(quats, log_scales, g, sh);
     const float mu[3] = {means[3 * (size_t)g], means[3 * (size_t)g + 1], means[3 * (size_t)g + 2]};
     GaussSums a = {};
+    bool seen = false;
     for (int v = 0; v < vt.n_views; ++v) {
         const size_t item = (size_t)v * n + g;
         const float4 a0 = acc_uvod[item], a1 = acc_conic[item];
         float tw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if ((a0.x != 0.f) | (a0.y != 0.f) | (a0.z != 0.f) | (a0.w != 0.f) | (a1.x != 0.f) | (a1.y != 0.f) | (a1.z != 0.f))
+        if ((a0.x != 0.f) | (a0.y != 0.f) | (a0.z != 0.f) | (a0.w != 0.f) | (a1.x != 0.f) | (a1.y != 0.f) | (a1.z != 0.f)) {
+            seen = true;
             project_view_bwd(vt, prm, pose_dev, v, mu, sh, a0, a1, pose, a, tw);
+        }
         if (pose) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) out.pose_part[((size_t)v * 6 + k) * n + g] = tw[k];
         }
     }
     if (!map) return;
-    write_gauss_grads(sh, a, logits[g], g, out);
+    if (seen) write_gauss_grads(sh, a, logits[g], g, out);
+    else write_no_grads(g, out);
     const float4 cr = acc_rgb[g];
     out.rgb[3 * (size_t)g] = cr.x;
     out.rgb[3 * (size_t)g + 1] = cr.y;

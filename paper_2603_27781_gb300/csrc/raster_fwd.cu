@@ -17,7 +17,9 @@ namespace {
 // pixels per thread: the blend loop is issue-bound, so warps resident matter
 // more than the few values ptxas would otherwise keep live across the mask flush.  At D = 16 with one
 // pixel per thread four CTAs rather than five (64 registers, 48): with 48 the loads of the two splats
-// evaluated together are taken apart (0.054 -> 0.044 ms at 320x240, 0.067 -> 0.056 at 64x48).
+// evaluated together are taken apart (0.054 -> 0.044 ms at 320x240, 0.067 -> 0.056 at 64x48).  At D = 16 with two
+// pixels per thread six CTAs (80 registers) spill 20 bytes, 36 in 16-bit storage; five take 0.241 ms
+// against 0.232 (1M Gaussians at 1200x680).
 constexpr int fwd_min_blocks(int D, int NP) {
     return NP == 1 ? (D == 0 ? 8 : D <= 4 ? 6 : D <= 8 ? 5 : D <= 16 ? 4 : 3) : NP == 2 ? (D <= 16 ? 6 : 4) : 6;
 }
@@ -322,8 +324,8 @@ __global__ void __launch_bounds__(Shape<NP>::THREADS, fwd_min_blocks(D, NP)) ras
 // its own shared memory, so it never waits at a barrier for the tile's other groups, and
 // it leaves as soon as its own pixels are done, freeing its registers and shared memory.
 // Arithmetic, order and outputs are those of raster_fwd_kernel.
-// Register caps that keep the blocks spill-free: 80 registers up to D = 16, 128 at D = 32 with two
-// pixels per thread.
+// Register caps: 80 registers with one pixel per thread, spill-free; with two, 80 at D = 16, where 20
+// bytes spill, and 128 at D = 32, spill-free.
 constexpr int fwd_group_min_blocks(int D, int NP) { return NP == 1 ? 24 : (D <= 16 ? 22 : 16); }
 
 template <int D, int NP, typename RT, typename FT>
@@ -676,9 +678,10 @@ extern "C" gs_status gs_render_fwd(const gs_gaussians *g, const gs_projected *pr
     // The default at D = 16 and 32 is two pixels per thread, and one where the image has too few tiles for
     // that: up to two waves of the two-pixel CTAs (six per SM at D = 16, four at D = 32) twice as many warps
     // hide more latency.  Measured, one against two pixels per thread: D = 16: 0.044 / 0.058 ms at 320x240, 0.068
-    // / 0.084 at 640x480, 0.145 / 0.156 (scan) at 800x600, then 0.103 / 0.098 at 880x600 and 0.237 / 0.218 at
-    // 1200x680; D = 32: 0.053 / 0.063 at 320x240, 0.148 / 0.163 at 640x480, but 0.114 / 0.109 at 811x607.  The
-    // images do not depend on it.
+    // / 0.084 at 640x480, then 0.103 / 0.098 at 880x600 and 0.237 / 0.218 at 1200x680; D = 32: 0.053 / 0.063
+    // at 320x240, 0.148 / 0.163 at 640x480, but 0.114 / 0.109 at 811x607.  A scanned map, whose splats are
+    // small, would take one pixel further: 0.145 / 0.156 at 800x600, which 1,900 tiles put just above the line of
+    // 1,824.  The images do not depend on it.
     if (!prm.fwd_np && g->feat_dim >= 16 && prm.fwd_blocks == GS_BWD_BLOCKS_DEFAULT && prm.fwd_batch == kBatch &&
         vt.tile_off[n_views] <= kSMs * (g->feat_dim == 16 ? 12 : 8))
         np = 1;

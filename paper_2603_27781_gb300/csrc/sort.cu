@@ -354,10 +354,11 @@ struct SortSmem {
 // One radix pass over BITS-wide digits, NT threads per block and IPT keys per thread: 256 threads for the
 // depth passes over the visible items, 512 with 8 or 16 keys for the tile passes over the instances.
 // Resident blocks per SM the register allocation must allow: four depth-pass blocks of 8 keys a
-// thread (64 registers), six of 4 (40); three tile-pass blocks of 8 (42 registers), two of 16 (64).  Whole binning in ms with
-// tile-pass blocks of 512 x 8 keys at three per SM, 1024 x 8 at two, 512 x 16 at two, 256 x 16 at four: 0.143 / 0.149 /
-// 0.146 / 0.149 (1M Gaussians at 1200x680, 1.7M instances), 0.091 / 0.098 / 0.096 / 0.096 (300k at 811x607),
-// 0.87 / 0.91 / 0.86 / 0.85 (2M, eight keyframes, 22M instances).
+// thread (64 registers), six of 4 (40); three tile-pass blocks of 8 (40 registers, 56 to 60 bytes spilled), two of
+// 16 (64 registers, 152 bytes spilled).  Whole binning in ms with tile-pass blocks of 512 x 8 keys at three per
+// SM, 1024 x 8 at two, 512 x 16 at two, 256 x 16 at four: 0.143 / 0.149 / 0.146 / 0.149 (1M Gaussians at 1200x680,
+// 1.7M instances), 0.091 / 0.098 / 0.096 / 0.096 (300k at 811x607), 0.87 / 0.91 / 0.86 / 0.85 (2M, eight
+// keyframes, 22M instances).
 template <int NT, int IPT> constexpr int sort_min_blocks() {
     return NT == 256 ? (IPT >= 8 ? 4 : 6) : (IPT >= 16 ? 2 : 3);
 }
